@@ -60,7 +60,11 @@ typedef enum {
 } tmnd_status;
 
 typedef enum {
-    TMND_F64 = 0,          /* FP64 storage and arithmetic: 24 complex128 planes per RHS */
+    TMND_F64 = 0,          /* FP64 storage: 24 complex128 planes per RHS.  The operator works on
+                              56-bit fixed-point copies with one exponent per site: results are as
+                              accurate as FP64 arithmetic relative to the largest component of the
+                              sites they are made of; a NaN or infinity makes all components of the
+                              sites it reaches NaN */
     TMND_F32 = 1,          /* FP32 storage: 24 complex64 planes per RHS */
     TMND_S16 = 2           /* 16-bit fixed-point storage with FP32 arithmetic, in blocks of
                               8 consecutive sites (800 bytes): 6 planes of 8 16-byte words
@@ -94,8 +98,8 @@ typedef struct tmnd_gauge tmnd_gauge;
 
 /* Create a gauge handle on the current CUDA device.  Copies `host_links`
  * (canonical layout, host memory, read only during the call) to the device
- * and packs it per parity and direction, in FP64 (18 reals per link) and in
- * 16-bit fixed point (rows 0 and 1, scale 32767; row 2 rebuilt in the
+ * and packs it per parity and direction, in 56-bit fixed point (18 reals per
+ * link, 8 bytes each), in FP32 and in 16-bit fixed point (rows 0 and 1, scale 32767; row 2 rebuilt in the
  * kernels) for the sloppy operator.  `prec` is TMND_F64 or TMND_S16 (both
  * copies are made either way).  Every link is checked on the host
  * to be SU(3) (|U U^+ - 1| and |det U - 1| below 1e-10); a failing link gives
@@ -137,7 +141,9 @@ tmnd_status tmnd_spinor_unpack(const tmnd_gauge *g, void *dev_canonical, const v
  * are TMND_F32 spinors and the operator is the FP32 one (one right-hand side
  * per launch sequence).  `out` and `in` must not overlap.  Uses
  * the handle's workspace (one even-site and one odd-site spinor per right-hand
- * side for TMND_OP_S16, one of each otherwise), growing it on first use.
+ * side for TMND_OP_S16; one of each for TMND_OP_F32, and for FP64 spinors on
+ * lattices that fill the chip: smaller ones get up to ~25000 sites' worth of
+ * each and run several right-hand sides per launch), growing it on first use.
  * (Sec. 2 even-odd Schur complement; Eq. "g5tau1-hermiticity".) */
 tmnd_status tm_nd_apply(tmnd_gauge *g, void *out, const void *in, int op, double sigma,
                         int nrhs, void *stream);
@@ -159,7 +165,7 @@ tmnd_status tm_nd_apply(tmnd_gauge *g, void *out, const void *in, int op, double
  *
  *   - Limit: V/2 <= TMND_NOALLOC_MAX_VH odd sites (e.g. 16^4, 8^3x64);
  *     larger lattices are rejected with TMND_ERR_ARG.  The array takes
- *     2 x 24 x TMND_NOALLOC_MAX_VH complex128 = 24 MiB on every GPU that loads
+ *     2 x 388 x TMND_NOALLOC_MAX_VH bytes = 24.25 MiB on every GPU that loads
  *     the library, until the process exits.
  *   - The current device must be the handle's device.
  *   - The first call on each device looks up the array's device address

@@ -7,7 +7,7 @@
 #include <complex>
 #include <vector>
 
-#include "tmnd_internal.cuh"
+#include "hop_fx.cuh"
 
 // ------------------------------------------------------------------ errors
 static thread_local char g_err[512] = "";
@@ -49,8 +49,8 @@ tmnd_status tmnd_ensure_partials(tmnd_gauge *g, size_t bytes) {
 }
 
 // ------------------------------------------------------------ link packing
-// canonical complex128 [4][T][X][Y][Z][3][3] -> [2 parity][4 mu][9][Vh]
-__global__ void k_pack_links(Geom g, const double2 *__restrict__ canon, double2 *__restrict__ out) {
+// canonical complex128 [4][T][X][Y][Z][3][3] -> FP32 [2 parity][4 mu][9][Vh]
+__global__ void k_pack_links_f32(Geom g, const double2 *__restrict__ canon, float2 *__restrict__ out) {
     long V = 2L * g.Vh;
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;  // over 4 * V * 9
     if (i >= 4 * V * 9) return;
@@ -65,7 +65,8 @@ __global__ void k_pack_links(Geom g, const double2 *__restrict__ canon, double2 
     int t = (int)(r / g.X);
     int par = (t + x + y + z) & 1;
     long h = lex >> 1;
-    out[(((size_t)par * 4 + mu) * 9 + k) * g.Vh + h] = canon[i];
+    const double2 u = canon[i];
+    out[(((size_t)par * 4 + mu) * 9 + k) * g.Vh + h] = make_float2((float)u.x, (float)u.y);
 }
 
 static bool su3_ok(const std::complex<double> *u) {
@@ -80,12 +81,6 @@ static bool su3_ok(const std::complex<double> *u) {
     std::complex<double> det = u[0] * (u[4] * u[8] - u[5] * u[7]) - u[1] * (u[3] * u[8] - u[5] * u[6]) +
                                u[2] * (u[3] * u[7] - u[4] * u[6]);
     return err < 1e-10 && std::abs(det - 1.0) < 1e-10;
-}
-
-// packed FP64 links -> the same layout in FP32 (the FP32 operator)
-__global__ void k_links_to_f32(long n, const double2 *__restrict__ in, float2 *__restrict__ out) {
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-        out[i] = make_float2((float)in[i].x, (float)in[i].y);
 }
 
 extern "C" tmnd_status tmnd_gauge_create(const double *host_links, const tmnd_action *act, int prec,
@@ -128,6 +123,7 @@ extern "C" tmnd_status tmnd_gauge_create(const double *host_links, const tmnd_ac
     g->st.kp = kp;
     g->st.kpp = kpp;
     g->st.inv_det = 1.0 / det;
+    g->fx = fx_site(g->st);
     g->stf.kappa2 = (float)g->st.kappa2;
     g->stf.kp = (float)kp;
     g->stf.kpp = (float)kpp;
@@ -135,23 +131,23 @@ extern "C" tmnd_status tmnd_gauge_create(const double *host_links, const tmnd_ac
 
     size_t nb = sizeof(double2) * 4 * V * 9;
     double2 *canon = nullptr;
-    cudaError_t e = cudaMalloc(&g->links, nb);
+    cudaError_t e = cudaMalloc(&g->links_fx, sizeof(int4) * fx_link_words(g->geom.Vh));
     if (e == cudaSuccess) e = cudaMalloc(&g->links_s16, sizeof(int2) * 3 * 4 * (size_t)V);
     if (e == cudaSuccess) e = cudaMalloc(&g->links_f32, sizeof(float2) * 4 * V * 9);
     if (e == cudaSuccess) e = cudaMalloc(&canon, nb);
     if (e == cudaSuccess) e = cudaMemcpy(canon, host_links, nb, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
         long n = 4 * V * 9;
-        k_pack_links<<<(unsigned)((n + 255) / 256), 256>>>(g->geom, canon, g->links);
+        launch_fx_pack_links(g->geom, canon, g->links_fx, 0);
         launch_pack_links_s16(g->geom, canon, g->links_s16, 0);
-        k_links_to_f32<<<(unsigned)((n + 255) / 256), 256>>>(n, g->links, g->links_f32);
+        k_pack_links_f32<<<(unsigned)((n + 255) / 256), 256>>>(g->geom, canon, g->links_f32);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (canon) cudaFree(canon);
     if (e != cudaSuccess) {
         tmnd_set_error("tmnd_gauge_create: %s", cudaGetErrorString(e));
-        if (g->links) cudaFree(g->links);
+        if (g->links_fx) cudaFree(g->links_fx);
         if (g->links_s16) cudaFree(g->links_s16);
         if (g->links_f32) cudaFree(g->links_f32);
         delete g;
@@ -164,7 +160,7 @@ extern "C" tmnd_status tmnd_gauge_create(const double *host_links, const tmnd_ac
 extern "C" void tmnd_gauge_destroy(tmnd_gauge *g) {
     if (!g) return;
     cudaDeviceSynchronize();
-    if (g->links) cudaFree(g->links);
+    if (g->links_fx) cudaFree(g->links_fx);
     if (g->links_s16) cudaFree(g->links_s16);
     if (g->links_f32) cudaFree(g->links_f32);
     if (g->work) cudaFree(g->work);
@@ -249,11 +245,35 @@ __global__ void k_g5tau1(int Vh, const double2 *__restrict__ in, double2 *__rest
     }
 }
 
-// Mhat (dag = false) or Mhat^+ applied to one right-hand side; te is an even-site temporary.
-static void apply_mhat(const tmnd_gauge *g, const double2 *in, double2 *out, double2 *te, bool dag,
-                       HopEpi epi, const HopEpiArgs &ea, cudaStream_t s) {
-    launch_hop_even_f64(g->geom, g->st, g->links, in, te, dag, nullptr, s);
-    launch_hop_odd_f64(g->geom, g->st, g->links, in, te, out, dag, epi, ea, s);
+// One operator application on FP64 right-hand sides, `batch` of them per launch.  work: 2 batch fixed-point
+// temporaries of fx_bytes each: the inputs' digits, then Mhat's results; the even-site intermediates.
+void apply_f64(const tmnd_gauge *g, double2 *out, const double2 *in, int op, double sigma, int nrhs, int batch,
+               void *work, cudaStream_t s) {
+    const int Vh = g->geom.Vh;
+    FxBatch bt;
+    bt.stride = fx_bytes(Vh);
+    bt.n64 = (size_t)NCOMP * Vh;
+    const FxOut a = fx_out(work, Vh), b = fx_next(a, batch * bt.stride);
+    const bool dag = op == TMND_OP_MHAT_DAG;
+    for (int k = 0; k < nrhs; k += batch) {
+        bt.nrhs = nrhs - k < batch ? nrhs - k : batch;
+        const double2 *ik = in + k * bt.n64;
+        FxOdd o = {};
+        o.out = a;
+        o.out64 = out + k * bt.n64;
+        launch_fx_from_f64(g->geom, ik, a, s, bt);
+        launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(a), b, dag, nullptr, s, bt);
+        if (op != TMND_OP_QHAT2) {
+            launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(a), fx_in(b), dag,
+                          op == TMND_OP_QHAT ? FX_F64_QHAT : FX_F64, o, s, bt);
+            continue;
+        }
+        launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(a), fx_in(b), false, FX_STORE, o, s, bt);
+        launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(a), b, true, nullptr, s, bt);
+        o.aux64 = ik;
+        o.sigma = sigma;
+        launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(a), fx_in(b), true, FX_F64_SHIFT, o, s, bt);
+    }
 }
 
 // Sloppy operator on TMND_S16 spinors: all right-hand sides in each stencil launch.
@@ -314,17 +334,17 @@ tmnd_status apply_f32(tmnd_gauge *g, float2 *out, const float2 *in, int op, doub
             case TMND_OP_MHAT:
             case TMND_OP_MHAT_DAG: {
                 const bool dag = op == TMND_OP_MHAT_DAG;
-                launch_hop_even_f32(g->geom, g->st, g->links_f32, ik, te, dag, nullptr, s);
+                launch_hop_even_f32(g->geom, g->st, g->links_f32, ik, te, dag, s);
                 launch_hop_odd_f32(g->geom, g->st, g->links_f32, ik, te, ok, dag, EPI_STORE, ea, s);
                 break;
             }
             case TMND_OP_QHAT2: {
-                launch_hop_even_f32(g->geom, g->st, g->links_f32, ik, te, false, nullptr, s);
+                launch_hop_even_f32(g->geom, g->st, g->links_f32, ik, te, false, s);
                 launch_hop_odd_f32(g->geom, g->st, g->links_f32, ik, te, yo, false, EPI_STORE, ea, s);
                 HopEpiArgsF e2 = {};
-                e2.sigma = sigma;
+                e2.sigma = (float)sigma;
                 e2.aux = ik;
-                launch_hop_even_f32(g->geom, g->st, g->links_f32, yo, te, true, nullptr, s);
+                launch_hop_even_f32(g->geom, g->st, g->links_f32, yo, te, true, s);
                 launch_hop_odd_f32(g->geom, g->st, g->links_f32, yo, te, ok, true, EPI_SHIFT, e2, s);
                 break;
             }
@@ -366,35 +386,12 @@ extern "C" tmnd_status tm_nd_apply(tmnd_gauge *g, void *out, const void *in, int
                    "tm_nd_apply: pointers must be 16-byte aligned");
     TMND_ARG_CHECK(isfinite(sigma), "tm_nd_apply: sigma must be finite");
     cudaGetLastError();  // clear a stale, non-sticky error left by earlier unrelated calls
-    const size_t sp = tmnd_spinor_bytes(g);
-    tmnd_status st = tmnd_ensure_workspace(g, 2 * sp);
+    // room for the largest batch from the first call on: a later call with more right-hand sides (under
+    // stream capture, say) does not allocate
+    const int batch = fx_batch(g->geom, nrhs);
+    tmnd_status st = tmnd_ensure_workspace(g, 2 * (size_t)fx_batch(g->geom, 1 << 30) * fx_bytes(g->geom.Vh));
     if (st != TMND_OK) return st;
-    double2 *te = (double2 *)g->work;
-    double2 *yo = (double2 *)((char *)g->work + sp);
-    cudaStream_t s = (cudaStream_t)stream;
-    const size_t n = sp / sizeof(double2);
-    HopEpiArgs ea = {};
-    for (int k = 0; k < nrhs; k++) {
-        const double2 *ik = (const double2 *)in + k * n;
-        double2 *ok = (double2 *)out + k * n;
-        switch (op) {
-            case TMND_OP_MHAT: apply_mhat(g, ik, ok, te, false, EPI_STORE, ea, s); break;
-            case TMND_OP_MHAT_DAG: apply_mhat(g, ik, ok, te, true, EPI_STORE, ea, s); break;
-            case TMND_OP_QHAT2: {
-                apply_mhat(g, ik, yo, te, false, EPI_STORE, ea, s);
-                HopEpiArgs e2 = {};
-                e2.sigma = sigma;
-                e2.aux = ik;
-                apply_mhat(g, yo, ok, te, true, EPI_SHIFT, e2, s);
-                break;
-            }
-            case TMND_OP_QHAT: {
-                apply_mhat(g, ik, yo, te, false, EPI_STORE, ea, s);
-                k_g5tau1<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g->geom.Vh, yo, ok);
-                break;
-            }
-        }
-    }
+    apply_f64(g, (double2 *)out, (const double2 *)in, op, sigma, nrhs, batch, g->work, (cudaStream_t)stream);
     TMND_CUDA_TRY(cudaGetLastError());
     return TMND_OK;
 }

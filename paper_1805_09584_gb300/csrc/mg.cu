@@ -294,8 +294,8 @@ __global__ void k_coarse_apply(MGGeom m, const float2 *__restrict__ Dc, const fl
 }
 
 // One direction of the single-flavour hop, w(x) = -kappa (1 -+ gamma_mu) U psi(x +- mu) (with the
-// antiperiodic sign), full lattice, FP32 with the FP64 links rounded on the fly.
-__global__ void k_hop_dir_f32(Geom g, double kappa, const double2 *__restrict__ links, const float2 *__restrict__ in,
+// antiperiodic sign), full lattice, FP32 links.
+__global__ void k_hop_dir_f32(Geom g, double kappa, const float2 *__restrict__ links, const float2 *__restrict__ in,
                               float2 *__restrict__ out, int d) {
     const int Vh = g.Vh;
     const int mu = d >> 1;
@@ -321,13 +321,13 @@ __global__ void k_hop_dir_f32(Geom g, double kappa, const double2 *__restrict__ 
         const int hn = ((c[0] * g.X + c[1]) * g.Y + c[2]) * g.Zh + (c[3] >> 1);
         const int Q = 1 - P;
         // link U_mu(x) (forward) at (P, h) or U_mu(x - mu) (backward) at (Q, hn)
-        const double2 *L = fwd ? links + ((size_t)(P * 4 + mu) * 9) * Vh : links + ((size_t)(Q * 4 + mu) * 9) * Vh;
+        const float2 *L = fwd ? links + ((size_t)(P * 4 + mu) * 9) * Vh : links + ((size_t)(Q * 4 + mu) * 9) * Vh;
         const int hl = fwd ? h : hn;
         float2 u[3][3];
         for (int a = 0; a < 3; a++)
             for (int bb = 0; bb < 3; bb++) {
-                const double2 w = L[(size_t)(a * 3 + bb) * Vh + hl];
-                u[a][bb] = fwd ? make_float2((float)w.x, (float)w.y) : make_float2((float)w.x, -(float)w.y);
+                const float2 w = L[(size_t)(a * 3 + bb) * Vh + hl];
+                u[a][bb] = fwd ? w : make_float2(w.x, -w.y);
             }
         float2 ps[4][3];
         for (int s = 0; s < 4; s++)
@@ -461,7 +461,7 @@ extern "C" tmnd_status tmnd_mg_create(tmnd_gauge *g, const tmnd_mg_params *p, co
         // identity part (P^+ P = 1) and Godd column
         k_mg_restrict<<<dim3(mg->nblock, 1), 256>>>(m, mg->P, col, 12, tmpc + (size_t)mg->nblock * n2 * 9, 9, 0);
         for (int dd = 0; dd < 8; dd++) {
-            k_hop_dir_f32<<<gb, 256>>>(g->geom, g->act.kappa, g->links, col, w, dd);
+            k_hop_dir_f32<<<gb, 256>>>(g->geom, g->act.kappa, g->links_f32, col, w, dd);
             // face of the hop direction -> neighbour block column; the rest -> self
             k_mg_restrict<<<dim3(mg->nblock, 1), 256>>>(m, mg->P, w, 12, tmpc + (size_t)mg->nblock * n2 * (1 + dd),
                                                         1 + dd, 0);

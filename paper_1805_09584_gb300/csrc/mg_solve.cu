@@ -22,10 +22,10 @@ tmnd_status launch_sap_color(const tmnd_gauge *g, const int bd[4], int color, do
 namespace {
 
 
-// Full-lattice doublet operator, output parity P, FP32 (links rounded from FP64):
+// Full-lattice doublet operator, output parity P, FP32:
 // y = (1 + i kp g5 t3 - kpp t1 [+ i s g5 t1 on odd sites]) x_P - kappa H x_{1-P}
 // nf = 2: doublet (24 components); nf = 1: one flavour, D_TM(+mu) (12 components, kpp and s ignored).
-__global__ void k_dnd_full(Geom g, double kappa, float kp, float kpp, float s_odd, const double2 *__restrict__ links,
+__global__ void k_dnd_full(Geom g, double kappa, float kp, float kpp, float s_odd, const float2 *__restrict__ links,
                            const float2 *__restrict__ in, float2 *__restrict__ out, int nf) {
     const int ncomp = 12 * nf;
     const int Vh = g.Vh;
@@ -56,13 +56,13 @@ __global__ void k_dnd_full(Geom g, double kappa, float kp, float kpp, float s_od
                 else c[mu]--;
             }
             const int hn = ((c[0] * g.X + c[1]) * g.Y + c[2]) * g.Zh + (c[3] >> 1);
-            const double2 *L = fwd ? links + ((size_t)(P * 4 + mu) * 9) * Vh : links + ((size_t)(Q * 4 + mu) * 9) * Vh;
+            const float2 *L = fwd ? links + ((size_t)(P * 4 + mu) * 9) * Vh : links + ((size_t)(Q * 4 + mu) * 9) * Vh;
             const int hl = fwd ? h : hn;
             float2 u[3][3];
             for (int a = 0; a < 3; a++)
                 for (int b = 0; b < 3; b++) {
-                    const double2 w = fwd ? L[(size_t)(a * 3 + b) * Vh + hl] : L[(size_t)(b * 3 + a) * Vh + hl];
-                    u[a][b] = fwd ? make_float2((float)w.x, (float)w.y) : make_float2((float)w.x, -(float)w.y);
+                    const float2 w = fwd ? L[(size_t)(a * 3 + b) * Vh + hl] : L[(size_t)(b * 3 + a) * Vh + hl];
+                    u[a][b] = fwd ? w : make_float2(w.x, -w.y);
                 }
             const float k = -(float)kappa * sg;
             for (int f = 0; f < nf; f++) {
@@ -233,7 +233,7 @@ struct MGSolver {
 
     void apply(const float2 *in, float2 *out) {
         k_dnd_full<<<nblk(n / 24), 256, 0, st>>>(g->geom, g->act.kappa, (float)g->st.kp, (float)g->st.kpp, (float)s,
-                                                g->links, in, out, 2);
+                                                g->links_f32, in, out, 2);
     }
     // smoothing of D' x = r from x = 0: nu SAP sweeps (each: per colour the residual of the
     // whole lattice, then block-local MR on the blocks of that colour), or nu MR steps
@@ -409,7 +409,7 @@ extern "C" tmnd_status tmnd_dnd_full_apply(tmnd_gauge *g, void *out, const void 
     TMND_ARG_CHECK(g && out && in && out != in, "tmnd_dnd_full_apply: bad arguments");
     cudaGetLastError();
     k_dnd_full<<<nblk(2L * g->geom.Vh), 256, 0, (cudaStream_t)stream>>>(
-        g->geom, g->act.kappa, (float)g->st.kp, (float)g->st.kpp, (float)s, g->links, (const float2 *)in,
+        g->geom, g->act.kappa, (float)g->st.kp, (float)g->st.kpp, (float)s, g->links_f32, (const float2 *)in,
         (float2 *)out, 2);
     TMND_CUDA_TRY(cudaGetLastError());
     return TMND_OK;
@@ -437,7 +437,7 @@ extern "C" tmnd_status tmnd_mg_smooth_vectors(tmnd_gauge *g, void *vecs, int nve
         float2 *x = (float2 *)vecs + (size_t)v * n;
         for (int k = 0; k < iters; k++) {
             k_dnd_full<<<nblk(2L * g->geom.Vh), 256, 0, st>>>(g->geom, g->act.kappa, (float)g->st.kp, 0.f, 0.f,
-                                                             g->links, x, t, 1);
+                                                             g->links_f32, x, t, 1);
             // r = -D x ; minimise |D (x + w r)| -> w = -(Dr... use the residual direction r = -Dx:
             // x <- x - w D x with w = <D x, x-ish>: plain MR on D x = 0: r = -D x, w = <D r, r>/<D r, D r>
             // (here r = -t and D r = -D t; the two signs cancel in w)

@@ -42,7 +42,7 @@
 #include <chrono>
 #include <vector>
 
-#include "tmnd_internal.cuh"
+#include "hop_fx.cuh"
 
 namespace {
 
@@ -53,6 +53,7 @@ struct MMSState {
     double rr;          // (r, r) at the start of the current iteration
     double bb;          // (b, b)
     double alpha_old, beta_old;
+    double alpha;       // of the current iteration (FP64 path, k_alpha)
     double zeta[NS], zeta_old[NS];
     int active[NS];
     int conv_iter[NS];
@@ -85,14 +86,13 @@ struct ShiftPtrsT {
 };
 using ShiftPtrs = ShiftPtrsT<double2>;
 
-__global__ void k_init(long n, const double2 *__restrict__ b, double2 *__restrict__ r, double2 *__restrict__ p,
-                       ShiftPtrs sp, int nshift, double *__restrict__ part) {
+__global__ void k_init(long n, const double2 *__restrict__ b, double2 *__restrict__ r, ShiftPtrs sp,
+                       int nshift, double *__restrict__ part) {
     __shared__ double red[40];
     double acc = 0.0;
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
         double2 v = b[i];
         r[i] = v;
-        p[i] = v;
         for (int s = 0; s < nshift; s++) {
             sp.p[s][i] = v;
             sp.x[s][i] = make_double2(0.0, 0.0);
@@ -151,15 +151,18 @@ __global__ void k_init_state_b(MMSState *st, size_t st_stride, const double *__r
 }
 
 // Scalar step of the recursion (one block; thread 0 does the arithmetic).
-// j = position of this iteration inside its window.
+// j = position of this iteration inside its window.  part_norm: partials of |y|^2, |p|^2 (NULL: st->alpha
+// is already that of this iteration).
 __device__ void scalars_step(MMSState *st, MMSCoef *cf, const double *__restrict__ part_norm, int nb_hop,
                              const double *__restrict__ part_rr, const MMSConst &c, int j, double *hist, int hist_cap,
                              double *red) {
     const int was_done = st->done;
     double yy = 0, pp = 0, rr_new = 0;
     if (!was_done) {
-        yy = block_reduce_partials(part_norm, nb_hop, red);
-        pp = block_reduce_partials(part_norm + nb_hop, nb_hop, red);
+        if (part_norm) {
+            yy = block_reduce_partials(part_norm, nb_hop, red);
+            pp = block_reduce_partials(part_norm + nb_hop, nb_hop, red);
+        }
         rr_new = block_reduce_partials(part_rr, nb_hop, red);
     }
     if (threadIdx.x != 0) return;
@@ -175,7 +178,7 @@ __device__ void scalars_step(MMSState *st, MMSCoef *cf, const double *__restrict
         cf->skip = 1;
         return;
     }
-    const double alpha = st->rr / (yy + c.sigma0 * pp);
+    const double alpha = part_norm ? st->rr / (yy + c.sigma0 * pp) : st->alpha;
     const double beta = rr_new / st->rr;
     if (!isfinite(alpha) || !isfinite(rr_new) || !isfinite(beta)) {
         st->status = TMND_ERR_NAN;
@@ -220,10 +223,19 @@ __device__ void scalars_step(MMSState *st, MMSCoef *cf, const double *__restrict
     if (!st->active[c.nsolve - 1] || it >= c.maxiter) st->done = 1;
 }
 
-__global__ void k_scalars(MMSState *st, MMSCoef *cf, const double *__restrict__ part_norm, int nb_hop,
-                          const double *__restrict__ part_rr, MMSConst c, int j, double *hist, int hist_cap) {
+__global__ void k_scalars(MMSState *st, MMSCoef *cf, int nb_hop, const double *__restrict__ part_rr, MMSConst c, int j,
+                          double *hist, int hist_cap) {
     __shared__ double red[40];
-    scalars_step(st, cf, part_norm, nb_hop, part_rr, c, j, hist, hist_cap, red);
+    scalars_step(st, cf, nullptr, nb_hop, part_rr, c, j, hist, hist_cap, red);
+}
+
+// alpha = (r, r) / (p, w), (p, w) = |Mhat p|^2 + sigma_0 |p|^2 from the partials of the first Mhat
+__global__ void k_alpha(MMSState *st, const double *__restrict__ part_norm, int nb_hop, double sigma0) {
+    __shared__ double red[40];
+    if (st->done) return;
+    const double yy = block_reduce_partials(part_norm, nb_hop, red);
+    const double pp = block_reduce_partials(part_norm + nb_hop, nb_hop, red);
+    if (threadIdx.x == 0) st->alpha = st->rr / (yy + sigma0 * pp);
 }
 
 // Batched: block k runs the scalar step of right-hand side k (state and
@@ -245,17 +257,6 @@ __global__ void k_all_done(const MMSState *st, size_t st_stride, int nrhs, int *
     int d = 1;
     for (int k = 0; k < nrhs; k++) d &= ((const MMSState *)((const char *)st + k * st_stride))->done;
     *done_all = d;
-}
-
-// p = r' + beta p (base search direction, every iteration)
-__global__ void k_pupdate(long n, const MMSCoef *__restrict__ cf, const double2 *__restrict__ r,
-                          double2 *__restrict__ p) {
-    if (cf->skip) return;
-    const double beta = cf->beta;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const double2 rv = r[i], pv = p[i];
-        p[i] = make_double2(fma(beta, pv.x, rv.x), fma(beta, pv.y, rv.y));
-    }
 }
 
 // Windowed multi-shift update (end of each window): for every shift active
@@ -322,15 +323,13 @@ __global__ void __launch_bounds__(UPD_THREADS) k_window(long n, const MMSCoef *_
     }
 }
 
-// |b - y|^2 partials (true residual)
-__global__ void k_diff_norm(long n, const double2 *__restrict__ b, const double2 *__restrict__ y,
-                            double *__restrict__ part) {
+// |b|^2 partials
+__global__ void k_norm2(long n, const double2 *__restrict__ b, double *__restrict__ part) {
     __shared__ double red[40];
     double acc = 0.0;
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        double2 u = b[i], v = y[i];
-        double dx = u.x - v.x, dy = u.y - v.y;
-        acc = fma(dx, dx, fma(dy, dy, acc));
+        const double2 u = b[i];
+        acc = fma(u.x, u.x, fma(u.y, u.y, acc));
     }
     double s = block_sum(acc, red);
     if (threadIdx.x == 0) part[blockIdx.x] = s;
@@ -463,22 +462,6 @@ __global__ void k_add_f32_to_f64(long n, const float2 *__restrict__ e, double2 *
         x[i] = v;
     }
 }
-
-// r = b - y in FP64 and block partials |r|^2 (true residual of the refinement)
-__global__ void k_resid(long n, const double2 *__restrict__ b, const double2 *__restrict__ y,
-                        double2 *__restrict__ r, double *__restrict__ part) {
-    __shared__ double red[40];
-    double acc = 0.0;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const double2 u = b[i], v = y[i];
-        const double2 d = make_double2(u.x - v.x, u.y - v.y);
-        r[i] = d;
-        acc = fma(d.x, d.x, fma(d.y, d.y, acc));
-    }
-    double t = block_sum(acc, red);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-}
-
 
 // ------------------------------------------------------------- hybrid helpers
 // out = in * (ar + i ai) + out (FP64 complex axpy)
@@ -630,10 +613,27 @@ tmnd_status run_graph_loop(cudaStream_t s, const int *done_dev, int maxiter, int
     return TMND_OK;
 }
 
+// r = b - (Qhat^2 + sigma) x in FP64, with fx_blocks() partials of |r|^2; fa, fb: fixed-point temporaries.
+void launch_fx_defect(const tmnd_gauge *g, const double2 *b, const double2 *x, double sigma, double2 *r, double *part,
+                      FxOut fa, FxOut fb, cudaStream_t s) {
+    FxOdd e = {};
+    e.out = fa;
+    launch_fx_from_f64(g->geom, x, fa, s);
+    launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(fa), fb, false, nullptr, s);
+    launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(fa), fx_in(fb), false, FX_STORE, e, s);
+    launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(fa), fb, true, nullptr, s);
+    e.b64 = b;
+    e.aux64 = x;
+    e.sigma = sigma;
+    e.r = r;
+    e.part_out = part;
+    launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(fa), fx_in(fb), true, FX_RESID, e, s);
+}
+
 }  // namespace
 
-// One right-hand side.  work holds the WIN residual slots, p, y, te, p_i[nshift]
-// (spinor-sized each).  Residual r^(k0+j+1) of window position j goes to slot
+// One right-hand side.  work holds the WIN residual slots and p_i[nshift] in FP64, then p, y and te as
+// fixed-point digits (hop_fx.cuh).  Residual r^(k0+j+1) of window position j goes to slot
 // j; position 0 reads slot WIN-1 (the last residual of the previous window,
 // or b at the start).
 static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *x, const double *sigma, int nshift,
@@ -647,16 +647,16 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
     RingPtrs ring;
     for (int l = 0; l < WIN; l++) ring.r[l] = slot[l] = (double2 *)(w + l * sp);
     double2 *r = slot[WIN - 1];
-    double2 *p = (double2 *)(w + (WIN + 0) * sp);
-    double2 *y = (double2 *)(w + (WIN + 1) * sp);
-    double2 *te = (double2 *)(w + (WIN + 2) * sp);
+    const int Vh = g->geom.Vh;
+    char *wx = w + (WIN + (size_t)nshift) * sp;
+    const FxOut p = fx_out(wx, Vh), y = fx_out(wx + fx_bytes(Vh), Vh), te = fx_out(wx + 2 * fx_bytes(Vh), Vh);
     ShiftPtrs ptrs = {};
     for (int i = 0; i < nshift; i++) {
         ptrs.x[i] = x[i] + (size_t)rhs_index * n;
-        ptrs.p[i] = (double2 *)(w + (WIN + 3 + i) * sp);
+        ptrs.p[i] = (double2 *)(w + (WIN + i) * sp);
     }
     // small device area after the partials
-    const int nb_hop = hop_blocks(g->geom);
+    const int nb_hop = fx_blocks(g->geom);
     const int nb_str = stream_blocks(n);
     double *part_norm = (double *)g->partials;              // 2 * nb_hop
     double *part_rr = part_norm + 2 * nb_hop;               // nb_hop
@@ -674,33 +674,34 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
     for (int i = 0; i < nshift; i++) c.delta[i] = sigma[i] - c.sigma0;
     c.rho2 = rho * rho;
 
-    k_init<<<nb_str, UPD_THREADS, 0, s>>>(n, b, r, p, ptrs, nshift, part_str);
+    k_init<<<nb_str, UPD_THREADS, 0, s>>>(n, b, r, ptrs, nshift, part_str);
+    launch_fx_from_f64(g->geom, b, p, s);
     k_init_state<<<1, 256, 0, s>>>(st, part_str, nb_str, c);
     TMND_CUDA_TRY(cudaGetLastError());
 
     auto body = [&](int k, auto mark) {
         const int j = k % WIN;  // position inside the window
         mark(0);
-        HopEpiArgs e1 = {};
+        FxOdd e1 = {};
+        e1.out = y;
         e1.part_out = part_norm;
         e1.done = &st->done;
-        launch_hop_even_f64(g->geom, g->st, g->links, p, te, false, &st->done, s);
-        launch_hop_odd_f64(g->geom, g->st, g->links, p, te, y, false, EPI_STORE_NORMS, e1, s);
-        launch_hop_even_f64(g->geom, g->st, g->links, y, te, true, &st->done, s);
-        HopEpiArgs e2 = {};
+        launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(p), te, false, &st->done, s);
+        launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(p), fx_in(te), false, FX_STORE_NORMS, e1, s);
+        k_alpha<<<1, 256, 0, s>>>(st, part_norm, nb_hop, c.sigma0);
+        launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(y), te, true, &st->done, s);
+        FxOdd e2 = {};
         e2.sigma = c.sigma0;
-        e2.aux = p;
+        e2.p = fx_in(p);
         e2.r_in = slot[(j + WIN - 1) % WIN];
         e2.r = slot[j];
+        e2.alpha = &st->alpha;
         e2.part_out = part_rr;
-        e2.part_in = part_norm;
-        e2.npart_in = nb_hop;
-        e2.rr = &st->rr;
         e2.done = &st->done;
-        launch_hop_odd_f64(g->geom, g->st, g->links, y, te, nullptr, true, EPI_MMS_R, e2, s);
+        launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(y), fx_in(te), true, FX_MMS_R, e2, s);
         mark(1);
-        k_scalars<<<1, 256, 0, s>>>(st, cf, part_norm, nb_hop, part_rr, c, j, hist, hist_cap);
-        k_pupdate<<<nb_str, UPD_THREADS, 0, s>>>(n, cf, slot[j], p);
+        k_scalars<<<1, 256, 0, s>>>(st, cf, nb_hop, part_rr, c, j, hist, hist_cap);
+        launch_fx_pupdate(g->geom, &cf->skip, &cf->beta, slot[j], p, s);
         if (j == WIN - 1) k_window<double2><<<nb_str, UPD_THREADS, 0, s>>>(n, cf, ring, ptrs, nshift);
         mark(2);
     };
@@ -710,7 +711,7 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
     const long nlaunch = lo.nlaunch;
     std::vector<float> &hop_t = lo.hop_t, &upd_t = lo.upd_t;
     if (info) {
-        info->launches += 2 + nlaunch * ((long long)check_every * 6 + check_every / WIN) + 5LL * nshift;
+        info->launches += 3 + nlaunch * ((long long)check_every * 7 + check_every / WIN) + 5LL * nshift;
         info->fp64_applies += nshift;
     }
 
@@ -727,25 +728,17 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
 
     // true residual |b - (Qhat^2 + sigma_i) x_i| / |b| with the operator; leaves the defect
     // b - (Qhat^2 + sigma_i) x_i in r
-    std::vector<double> hpart(nb_str);
+    std::vector<double> hpart(nb_hop);
     auto true_res_of = [&](int i, double *tr) -> tmnd_status {
-        HopEpiArgs ea = {};
-        launch_hop_even_f64(g->geom, g->st, g->links, ptrs.x[i], te, false, nullptr, s);
-        launch_hop_odd_f64(g->geom, g->st, g->links, ptrs.x[i], te, r, false, EPI_STORE, ea, s);
-        HopEpiArgs e2 = {};
-        e2.sigma = sigma[i];
-        e2.aux = ptrs.x[i];
-        launch_hop_even_f64(g->geom, g->st, g->links, r, te, true, nullptr, s);
-        launch_hop_odd_f64(g->geom, g->st, g->links, r, te, y, true, EPI_SHIFT, e2, s);
-        k_resid<<<nb_str, UPD_THREADS, 0, s>>>(n, b, y, r, part_str);
-        cudaError_t e3 = cudaMemcpyAsync(hpart.data(), part_str, sizeof(double) * nb_str, cudaMemcpyDeviceToHost, s);
+        launch_fx_defect(g, b, ptrs.x[i], sigma[i], r, part_rr, p, te, s);
+        cudaError_t e3 = cudaMemcpyAsync(hpart.data(), part_rr, sizeof(double) * nb_hop, cudaMemcpyDeviceToHost, s);
         if (e3 == cudaSuccess) e3 = cudaStreamSynchronize(s);
         if (e3 != cudaSuccess) {
             tmnd_set_error("mms_cg_solve: %s", cudaGetErrorString(e3));
             return TMND_ERR_CUDA;
         }
         double acc = 0;
-        for (int k = 0; k < nb_str; k++) acc += hpart[k];
+        for (int k = 0; k < nb_hop; k++) acc += hpart[k];
         *tr = hs.bb > 0 ? sqrt(acc / hs.bb) : 0.0;
         return TMND_OK;
     };
@@ -819,7 +812,8 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
 // Workspace of the mixed solve: FP64 vectors for one right-hand side at a time
 // (defect correction), sloppy vectors for nrhs right-hand sides at once.
 struct MixedWork {
-    double2 *r64, *y64, *te64;          // FP64: defect, (Qhat^2+sigma) x, even temporary
+    double2 *r64;                       // FP64 defect
+    FxOut fa, fb;                       // fixed-point temporaries of the FP64 operator
     SloppyVecs v;                       // FP32 ring, b, p_i, x_i and the 16-bit p (nrhs blocks)
     void *y16, *te16;                   // 16-bit stencil temporaries, nrhs blocks of v.sb
     int nrhs;
@@ -838,7 +832,7 @@ struct MixedWork {
 static size_t mixed_work_bytes(int Vh, int nshift, int nrhs = 1) {
     const size_t s64 = spinor_bytes_prec(Vh, TMND_F64), s32 = spinor_bytes_prec(Vh, TMND_F32),
                  s16 = spinor_bytes_prec(Vh, TMND_S16);
-    return 3 * s64 + (size_t)nrhs * ((WIN + 1 + 2 * (size_t)nshift) * s32 + 3 * s16);
+    return s64 + 2 * fx_bytes(Vh) + (size_t)nrhs * ((WIN + 1 + 2 * (size_t)nshift) * s32 + 3 * s16);
 }
 
 static MixedWork mixed_work(void *base, int Vh, int nshift, int nrhs = 1) {
@@ -847,8 +841,8 @@ static MixedWork mixed_work(void *base, int Vh, int nshift, int nrhs = 1) {
     char *w = (char *)base;
     MixedWork m;
     m.r64 = (double2 *)w; w += s64;
-    m.y64 = (double2 *)w; w += s64;
-    m.te64 = (double2 *)w; w += s64;
+    m.fa = fx_out(w, Vh); w += fx_bytes(Vh);
+    m.fb = fx_out(w, Vh); w += fx_bytes(Vh);
     m.v.n = 24L * Vh;
     m.v.sb = s16;
     m.v.nshift = nshift;
@@ -987,18 +981,9 @@ static size_t sloppy_partial_bytes(const Geom &geom, int nrhs) {
 // (Qhat^2 + sigma) x - b in FP64 into m.r64 (as b - (...)), returns |r|^2 on the host.
 static tmnd_status fp64_defect(tmnd_gauge *g, const MixedWork &m, const double2 *b, const double2 *x, double sigma,
                                cudaStream_t s, double *rr) {
-    const long n = 24L * g->geom.Vh;
-    const int nb = stream_blocks(n);
+    const int nb = fx_blocks(g->geom);
     double *part = (double *)g->partials;
-    HopEpiArgs ea = {};
-    launch_hop_even_f64(g->geom, g->st, g->links, x, m.te64, false, nullptr, s);
-    launch_hop_odd_f64(g->geom, g->st, g->links, x, m.te64, m.r64, false, EPI_STORE, ea, s);
-    HopEpiArgs e2 = {};
-    e2.sigma = sigma;
-    e2.aux = x;
-    launch_hop_even_f64(g->geom, g->st, g->links, m.r64, m.te64, true, nullptr, s);
-    launch_hop_odd_f64(g->geom, g->st, g->links, m.r64, m.te64, m.y64, true, EPI_SHIFT, e2, s);
-    k_resid<<<nb, UPD_THREADS, 0, s>>>(n, b, m.y64, m.r64, part);
+    launch_fx_defect(g, b, x, sigma, m.r64, part, m.fa, m.fb, s);
     std::vector<double> h(nb);
     TMND_CUDA_TRY(cudaMemcpyAsync(h.data(), part, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
     TMND_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1254,8 +1239,7 @@ static tmnd_status mixed_batch(tmnd_gauge *g, const double2 *b, double2 *const *
     for (int k = 0; k < R; k++) {
         const int nb = stream_blocks(n);
         double *part = (double *)g->partials;
-        TMND_CUDA_TRY(cudaMemsetAsync(m.y64, 0, sizeof(double2) * n, s));
-        k_diff_norm<<<nb, UPD_THREADS, 0, s>>>(n, b + (size_t)(k0 + k) * n, m.y64, part);
+        k_norm2<<<nb, UPD_THREADS, 0, s>>>(n, b + (size_t)(k0 + k) * n, part);
         std::vector<double> h(nb);
         TMND_CUDA_TRY(cudaMemcpyAsync(h.data(), part, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
         TMND_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1374,11 +1358,11 @@ extern "C" tmnd_status mms_cg_solve(tmnd_gauge *g, const void *b, int nrhs, cons
     if (R > nrhs) R = nrhs;
     const size_t sp = tmnd_spinor_bytes(g);
     tmnd_status st = tmnd_ensure_workspace(
-        g, mixed ? mixed_total_bytes(g->geom.Vh, nshift, nsolve, R) : (WIN + 3 + (size_t)nshift) * sp);
+        g, mixed ? mixed_total_bytes(g->geom.Vh, nshift, nsolve, R) : (WIN + (size_t)nshift) * sp + 3 * fx_bytes(g->geom.Vh));
     if (st != TMND_OK) return st;
     const long n = (long)(sp / sizeof(double2));
-    const int nbh = hop_blocks(g->geom) > hop_blocks_s16_max(g->geom) ? hop_blocks(g->geom)
-                                                                       : hop_blocks_s16_max(g->geom);
+    const int nbh = fx_blocks(g->geom) > hop_blocks_s16_max(g->geom) ? fx_blocks(g->geom)
+                                                                      : hop_blocks_s16_max(g->geom);
     const int nbs = stream_blocks(n) > site_blocks(g->geom.Vh) ? stream_blocks(n) : site_blocks(g->geom.Vh);
     size_t pbytes = sizeof(double) * (3 * (size_t)nbh + nbs) + 256 + 2 * 4096 + sizeof(MMSState) + sizeof(MMSCoef);
     if (mixed) {
@@ -1541,13 +1525,15 @@ extern "C" tmnd_status tmnd_hybrid_solve(tmnd_gauge *g, tmnd_mg *mg, const void 
     if (st != TMND_OK) return st;
     const long nfull = 2 * n;  // full-lattice FP32 doublet (complex numbers)
     const size_t f32b = sizeof(float2) * nfull;
-    const size_t scratch_b = 3 * sp + 4 * f32b + (mg ? mg_gcr_scratch_bytes(mg, hp->mg_restart > 0 ? hp->mg_restart : 24) : 0);
+    const size_t fxb = fx_bytes(Vh);
+    const size_t scratch_b = 2 * fxb + sp + 4 * f32b + (mg ? mg_gcr_scratch_bytes(mg, hp->mg_restart > 0 ? hp->mg_restart : 24) : 0);
     char *scr = nullptr;
     TMND_CUDA_TRY(cudaMalloc(&scr, scratch_b));
-    double2 *tq = (double2 *)scr, *te = (double2 *)(scr + sp), *gb = (double2 *)(scr + 2 * sp);
-    float2 *rhs = (float2 *)(scr + 3 * sp), *yp = (float2 *)(scr + 3 * sp + f32b);
-    float2 *ym = (float2 *)(scr + 3 * sp + 2 * f32b);
-    void *gcr = scr + 3 * sp + 4 * f32b;
+    const FxOut fa = fx_out(scr, Vh), fb = fx_out(scr + fxb, Vh);
+    double2 *gb = (double2 *)(scr + 2 * fxb);
+    char *sf = scr + 2 * fxb + sp;
+    float2 *rhs = (float2 *)sf, *yp = (float2 *)(sf + f32b), *ym = (float2 *)(sf + 2 * f32b);
+    void *gcr = sf + 4 * f32b;
     // private stream ordered after the caller's (the defect correction captures graphs,
     // which the legacy default stream does not allow)
     cudaStream_t user = (cudaStream_t)stream;
@@ -1567,8 +1553,7 @@ extern "C" tmnd_status tmnd_hybrid_solve(tmnd_gauge *g, tmnd_mg *mg, const void 
     std::vector<double> bbk(nrhs, 0.0);
     for (int k = 0; k < nrhs && res_status == TMND_OK; k++) {
         double *part = (double *)g->partials;
-        cudaMemsetAsync(m.y64, 0, sizeof(double2) * n, s);
-        k_diff_norm<<<nbs, UPD_THREADS, 0, s>>>(n, (const double2 *)b + (size_t)k * n, m.y64, part);
+        k_norm2<<<nbs, UPD_THREADS, 0, s>>>(n, (const double2 *)b + (size_t)k * n, part);
         std::vector<double> h(nbs);
         cudaMemcpyAsync(h.data(), part, sizeof(double) * nbs, cudaMemcpyDeviceToHost, s);
         cudaError_t e = cudaStreamSynchronize(s);
@@ -1647,14 +1632,16 @@ extern "C" tmnd_status tmnd_hybrid_solve(tmnd_gauge *g, tmnd_mg *mg, const void 
                 for (int sgn = 1; sgn >= -1; sgn -= 2) {
                     float2 *y = sgn > 0 ? yp : ym;
                     // odd guess (Qhat - sgn i s) x~ ; Qhat = g5 t1 Mhat
-                    HopEpiArgs ea = {};
-                    launch_hop_even_f64(g->geom, g->st, g->links, xk[i], te, false, nullptr, s);
-                    launch_hop_odd_f64(g->geom, g->st, g->links, xk[i], te, tq, false, EPI_STORE, ea, s);
-                    k_g5tau1<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(Vh, tq, gb);
+                    FxOdd e = {};
+                    e.out64 = gb;
+                    launch_fx_from_f64(g->geom, xk[i], fa, s);
+                    launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(fa), fb, false, nullptr, s);
+                    launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(fa), fx_in(fb), false, FX_F64_QHAT, e, s);
                     k_zaxpy64<<<nbs, 256, 0, s>>>(n, 0.0, -sgn * sq, xk[i], gb);
                     // even part eliminated: x_e = -D_ee^-1 D_eo x_o = kappa A^-1 H x_o = t_e / kappa
-                    launch_hop_even_f64(g->geom, g->st, g->links, gb, te, false, nullptr, s);
-                    k_to_f32_scaled<<<nbs, 256, 0, s>>>(n, 1.0 / g->act.kappa, te, y);
+                    launch_fx_from_f64(g->geom, gb, fa, s);
+                    launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(fa), fb, false, nullptr, s);
+                    launch_fx_to_f32(g->geom, 1.0 / g->act.kappa, fx_in(fb), y, s);
                     k_to_f32_scaled<<<nbs, 256, 0, s>>>(n, 1.0, gb, y + n);
                     int it = 0;
                     double rres = 0;

@@ -10,26 +10,27 @@
 // device-wide synchronisation of cudaMalloc/cudaFree.
 #include <mutex>
 
-#include "tmnd_internal.cuh"
+#include "hop_fx.cuh"
 
-// Scratch: the even-site temporary followed by the odd-site temporary, each
-// 24 complex128 planes of at most TMND_NOALLOC_MAX_VH sites (24 MiB total).
+// Scratch: two fixed-point spinors (hop_fx.cuh) of at most TMND_NOALLOC_MAX_VH sites, 24 planes of
+// 16-byte words and an exponent per site each (24.25 MiB total).
 // Every GPU that loads the library holds this array until the process exits.
-static __device__ __align__(256) double2 g_noalloc_scratch[2 * NCOMP * TMND_NOALLOC_MAX_VH];
+constexpr size_t SCRATCH_SPINOR = (size_t)TMND_NOALLOC_MAX_VH * (NCOMP * sizeof(int4) + sizeof(int));
+static __device__ __align__(256) char g_noalloc_scratch[2 * SCRATCH_SPINOR];
 
-// gamma_5 tau_1 kernel of the allocating path (defined in gauge.cu).
-__global__ void k_g5tau1(int Vh, const double2 *__restrict__ in, double2 *__restrict__ out);
+void apply_f64(const tmnd_gauge *g, double2 *out, const double2 *in, int op, double sigma, int nrhs, int batch,
+               void *work, cudaStream_t s);  // gauge.cu
 
 namespace {
 
 constexpr int MAX_DEVICES = 64;
 std::mutex g_mutex;
-double2 *g_scratch_addr[MAX_DEVICES] = {};
+char *g_scratch_addr[MAX_DEVICES] = {};
 
 // Device address of the scratch array on the current device.  In host code
 // `g_noalloc_scratch` names a host-side shadow, not device memory, so the
 // address is looked up once per device with that device current.
-tmnd_status scratch_address(double2 **out) {
+tmnd_status scratch_address(char **out) {
     int dev = 0;
     TMND_CUDA_TRY(cudaGetDevice(&dev));
     TMND_ARG_CHECK(dev >= 0 && dev < MAX_DEVICES, "tm_nd_apply_noalloc: device ordinal %d out of range", dev);
@@ -42,7 +43,7 @@ tmnd_status scratch_address(double2 **out) {
                            dev, cudaGetErrorString(e));
             return TMND_ERR_CUDA;
         }
-        g_scratch_addr[dev] = (double2 *)p;
+        g_scratch_addr[dev] = (char *)p;
     }
     *out = g_scratch_addr[dev];
     return TMND_OK;
@@ -66,47 +67,17 @@ extern "C" tmnd_status tm_nd_apply_noalloc(const tmnd_gauge *g, void *out, const
     TMND_CUDA_TRY(cudaGetDevice(&dev));
     TMND_ARG_CHECK(dev == g->device, "tm_nd_apply_noalloc: current device %d is not the handle's device %d", dev,
                    g->device);
-    double2 *scratch = nullptr;
+    char *scratch = nullptr;
     tmnd_status st = scratch_address(&scratch);
     if (st != TMND_OK) return st;
     cudaGetLastError();  // clear a stale, non-sticky error left by earlier unrelated calls
 
     // Both temporaries are fully written before they are read, so nothing
     // needs clearing between calls.
-    const size_t n = (size_t)NCOMP * g->geom.Vh;
-    double2 *te = scratch;
-    double2 *yo = scratch + n;
-    cudaStream_t s = (cudaStream_t)stream;
-    HopEpiArgs ea = {};
-    for (int k = 0; k < nrhs; k++) {
-        const double2 *ik = (const double2 *)in + k * n;
-        double2 *ok = (double2 *)out + k * n;
-        switch (op) {
-            case TMND_OP_MHAT:
-            case TMND_OP_MHAT_DAG: {
-                const bool dag = op == TMND_OP_MHAT_DAG;
-                launch_hop_even_f64(g->geom, g->st, g->links, ik, te, dag, nullptr, s);
-                launch_hop_odd_f64(g->geom, g->st, g->links, ik, te, ok, dag, EPI_STORE, ea, s);
-                break;
-            }
-            case TMND_OP_QHAT2: {
-                launch_hop_even_f64(g->geom, g->st, g->links, ik, te, false, nullptr, s);
-                launch_hop_odd_f64(g->geom, g->st, g->links, ik, te, yo, false, EPI_STORE, ea, s);
-                HopEpiArgs e2 = {};
-                e2.sigma = sigma;
-                e2.aux = ik;
-                launch_hop_even_f64(g->geom, g->st, g->links, yo, te, true, nullptr, s);
-                launch_hop_odd_f64(g->geom, g->st, g->links, yo, te, ok, true, EPI_SHIFT, e2, s);
-                break;
-            }
-            case TMND_OP_QHAT: {
-                launch_hop_even_f64(g->geom, g->st, g->links, ik, te, false, nullptr, s);
-                launch_hop_odd_f64(g->geom, g->st, g->links, ik, te, yo, false, EPI_STORE, ea, s);
-                k_g5tau1<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g->geom.Vh, yo, ok);
-                break;
-            }
-        }
-    }
+    int batch = fx_batch(g->geom, nrhs);
+    const int room = (int)(SCRATCH_SPINOR / fx_bytes(g->geom.Vh));
+    batch = batch < room ? batch : room;
+    apply_f64(g, (double2 *)out, (const double2 *)in, op, sigma, nrhs, batch, scratch, (cudaStream_t)stream);
     TMND_CUDA_TRY(cudaGetLastError());
     return TMND_OK;
 }

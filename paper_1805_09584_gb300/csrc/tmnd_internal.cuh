@@ -51,6 +51,14 @@ struct SiteTermF {
     float kappa2, kp, kpp, inv_det;
 };
 
+// Site term digits: kappa^2 A^-1 = (a, b = a kp, c = a kpp) 2^inv_e on even sites and
+// A = (1, kp, -kpp) 2^fwd_e on odd ones; |a| + |b| + |c| <= 1 in these units, so an output's
+// exponent is the input's plus inv_e or fwd_e.
+struct FxSite {
+    int2 inv_a, inv_b, inv_c, fwd_a, fwd_b, fwd_c;
+    int inv_e, fwd_e;
+};
+
 // Gauge handle.
 struct tmnd_gauge {
     tmnd_action act;
@@ -58,8 +66,9 @@ struct tmnd_gauge {
     int device;
     Geom geom;
     SiteTerm st;
-    double2 *links;        // [2 parity][4 mu][9][Vh] complex, U_mu(x) stored at the parity/half-index of x
-    float2 *links_f32;     // the same in FP32 (the FP32 operator)
+    int4 *links_fx;        // [2 parity][4 mu] in two digits, runs of 16 sites (hop_fx.cuh), U_mu(x) at x's parity/half-index
+    FxSite fx;             // digits of the site term
+    float2 *links_f32;     // [2 parity][4 mu][9][Vh] in FP32 (the FP32 operator, the multigrid)
     int2 *links_s16;       // [2 parity][4 mu][3][Vh]: rows 0, 1 as int16 pairs (scale 32767)
     SiteTermF stf;         // FP32 copy of st for the sloppy kernels
     void *work;            // grow-only workspace
@@ -75,38 +84,9 @@ tmnd_status tmnd_ensure_partials(tmnd_gauge *g, size_t bytes);
 constexpr int NCOMP = 24;
 
 // --------------------------------------------------------- device helpers
-__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-// i * a
-__device__ __forceinline__ double2 cmuli(double2 a) { return make_double2(-a.y, a.x); }
-// -i * a
-__device__ __forceinline__ double2 cmulmi(double2 a) { return make_double2(a.y, -a.x); }
 __device__ __forceinline__ double2 cneg(double2 a) { return make_double2(-a.x, -a.y); }
-// acc + a*b
-__device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 acc) {
-    return make_double2(fma(a.x, b.x, fma(-a.y, b.y, acc.x)), fma(a.x, b.y, fma(a.y, b.x, acc.y)));
-}
-// a*b
-__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-    return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
-}
-// acc + conj(a)*b
-__device__ __forceinline__ double2 cfma_conj(double2 a, double2 b, double2 acc) {
-    return make_double2(fma(a.x, b.x, fma(a.y, b.y, acc.x)), fma(a.x, b.y, fma(-a.y, b.x, acc.y)));
-}
-// conj(a)*b
-__device__ __forceinline__ double2 cmul_conj(double2 a, double2 b) {
-    return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.x, b.y, -a.y * b.x));
-}
-// Flip the sign of a double without touching the FP64 pipe (integer XOR of the sign bit).
-__device__ __forceinline__ double dflip(double v, unsigned long long mask) {
-    return __longlong_as_double(__double_as_longlong(v) ^ (long long)mask);
-}
-__device__ __forceinline__ double2 cflip(double2 a, unsigned long long mask) {
-    return make_double2(dflip(a.x, mask), dflip(a.y, mask));
-}
 
-// The same complex helpers in FP32 (the FP32 instantiation of the FP64 stencil).
+// Complex helpers in FP32.
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 cmuli(float2 a) { return make_float2(-a.y, a.x); }
@@ -159,7 +139,7 @@ __device__ __forceinline__ double block_reduce_partials(const double *p, int n, 
 }
 
 // --------------------------------------------------------- launch helpers
-// Hop kernels (tm_nd_apply and the solver share these launchers).
+// Epilogues of the FP32 and 16-bit odd-site kernels (tm_nd_apply and the solver share the launchers).
 enum HopEpi {
     EPI_STORE = 0,        // out = y
     EPI_STORE_NORMS = 1,  // out = y; partials |y|^2, |in|^2
@@ -169,37 +149,17 @@ enum HopEpi {
 
 constexpr int HOP_THREADS = 128;
 
-template <typename C2>
-struct HopEpiT {
-    double sigma;
-    const C2 *aux;          // EPI_SHIFT / EPI_MMS_R: the vector multiplied by sigma
-    C2 *r;                  // EPI_MMS_R: updated residual (written)
-    const C2 *r_in;         // EPI_MMS_R: residual before the update (NULL: update r in place)
-    double *part_out;       // partial sums written per block (EPI_STORE_NORMS: 2 per block; EPI_MMS_R: 1)
-    const double *part_in;  // EPI_MMS_R: partials of |y|^2, |p|^2 from the previous kernel
-    int npart_in;           // number of blocks that wrote part_in
-    const double *rr;       // EPI_MMS_R: (r,r) before the update (device scalar)
-    const int *done;        // if non-null and *done != 0 the kernel returns immediately
+struct HopEpiArgsF {
+    float sigma;
+    const float2 *aux;      // EPI_SHIFT: the vector multiplied by sigma
 };
-using HopEpiArgs = HopEpiT<double2>;
-using HopEpiArgsF = HopEpiT<float2>;
 
-// even-site kernel: t_e = kappa^2 A^-1 H_eo psi_o   (dag: kappa^2 A(-mu)^-1 H_eo gamma_5 psi_o)
-void launch_hop_even_f64(const Geom &g, const SiteTerm &st, const double2 *links, const double2 *psi_o,
-                         double2 *t_e, bool dag, const int *done, cudaStream_t s);
-// odd-site kernel: y_o = A psi_o - H_oe t_e   (dag: A(-mu) psi_o - gamma_5 H_oe t_e), with epilogue
-void launch_hop_odd_f64(const Geom &g, const SiteTerm &st, const double2 *links, const double2 *psi_o,
-                        const double2 *t_e, double2 *y_o, bool dag, HopEpi epi, const HopEpiArgs &ea,
-                        cudaStream_t s);
-// Number of blocks (= reduction partials) of every hop launch for this geometry.
-int hop_blocks(const Geom &g);
-// The same stencil in FP32 on FP32 planes with 18-real FP32 links (the FP32 operator:
+// The stencil in FP32 on FP32 planes with 18-real FP32 links (the FP32 operator:
 // accurate to ~1e-7, used for inner residuals of the defect correction)
 void launch_hop_even_f32(const Geom &g, const SiteTerm &st, const float2 *links, const float2 *psi_o, float2 *t_e,
-                         bool dag, const int *done, cudaStream_t s);
+                         bool dag, cudaStream_t s);
 void launch_hop_odd_f32(const Geom &g, const SiteTerm &st, const float2 *links, const float2 *psi_o,
                         const float2 *t_e, float2 *y_o, bool dag, HopEpi epi, const HopEpiArgsF &ea, cudaStream_t s);
-int hop_blocks_f32(const Geom &g);
 
 // ------------------------------------------------- sloppy (16-bit) path
 
