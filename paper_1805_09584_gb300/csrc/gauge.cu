@@ -321,37 +321,29 @@ static tmnd_status apply_s16(tmnd_gauge *g, void *out, const void *in, int op, d
     return TMND_OK;
 }
 
-// FP32 operator on TMND_F32 spinors (24 complex64 planes per right-hand side), one
-// right-hand side per launch sequence.
-tmnd_status apply_f32(tmnd_gauge *g, float2 *out, const float2 *in, int op, double sigma, int nrhs, float2 *te,
-                      float2 *yo, cudaStream_t s) {
+// FP32 operator on TMND_F32 spinors (24 complex64 planes per right-hand side), `batch` right-hand sides per
+// launch; te, yo: batch spinors each.
+tmnd_status apply_f32(tmnd_gauge *g, float2 *out, const float2 *in, int op, double sigma, int nrhs, int batch,
+                      float2 *te, float2 *yo, cudaStream_t s) {
+    TMND_ARG_CHECK(op == TMND_OP_MHAT || op == TMND_OP_MHAT_DAG || op == TMND_OP_QHAT2,
+                   "tm_nd_apply: op %d not available for TMND_F32 spinors", op);
     const size_t n = (size_t)NCOMP * g->geom.Vh;
-    HopEpiArgsF ea = {};
-    for (int k = 0; k < nrhs; k++) {
+    const bool dag = op == TMND_OP_MHAT_DAG;
+    for (int k = 0; k < nrhs; k += batch) {
+        const int r = nrhs - k < batch ? nrhs - k : batch;
         const float2 *ik = in + k * n;
         float2 *ok = out + k * n;
-        switch (op) {
-            case TMND_OP_MHAT:
-            case TMND_OP_MHAT_DAG: {
-                const bool dag = op == TMND_OP_MHAT_DAG;
-                launch_hop_even_f32(g->geom, g->st, g->links_f32, ik, te, dag, s);
-                launch_hop_odd_f32(g->geom, g->st, g->links_f32, ik, te, ok, dag, EPI_STORE, ea, s);
-                break;
-            }
-            case TMND_OP_QHAT2: {
-                launch_hop_even_f32(g->geom, g->st, g->links_f32, ik, te, false, s);
-                launch_hop_odd_f32(g->geom, g->st, g->links_f32, ik, te, yo, false, EPI_STORE, ea, s);
-                HopEpiArgsF e2 = {};
-                e2.sigma = (float)sigma;
-                e2.aux = ik;
-                launch_hop_even_f32(g->geom, g->st, g->links_f32, yo, te, true, s);
-                launch_hop_odd_f32(g->geom, g->st, g->links_f32, yo, te, ok, true, EPI_SHIFT, e2, s);
-                break;
-            }
-            default:
-                tmnd_set_error("tm_nd_apply: op %d not available for TMND_F32 spinors", op);
-                return TMND_ERR_ARG;
+        HopEpiArgsF ea = {};
+        launch_hop_even_f32(g->geom, g->st, g->links_f32, ik, te, dag, r, s);
+        if (op != TMND_OP_QHAT2) {
+            launch_hop_odd_f32(g->geom, g->st, g->links_f32, ik, te, ok, dag, EPI_STORE, ea, r, s);
+            continue;
         }
+        launch_hop_odd_f32(g->geom, g->st, g->links_f32, ik, te, yo, false, EPI_STORE, ea, r, s);
+        launch_hop_even_f32(g->geom, g->st, g->links_f32, yo, te, true, r, s);
+        ea.sigma = (float)sigma;
+        ea.aux = ik;
+        launch_hop_odd_f32(g->geom, g->st, g->links_f32, yo, te, ok, true, EPI_SHIFT, ea, r, s);
     }
     TMND_CUDA_TRY(cudaGetLastError());
     return TMND_OK;
@@ -367,10 +359,13 @@ extern "C" tmnd_status tm_nd_apply(tmnd_gauge *g, void *out, const void *in, int
                        "tm_nd_apply: bad arguments (FP32 spinors)");
         cudaGetLastError();
         const size_t s32 = spinor_bytes_prec(g->geom.Vh, TMND_F32);
-        tmnd_status st = tmnd_ensure_workspace(g, 2 * s32);
+        // as for FP64 spinors: small lattices run several right-hand sides per launch, and have the room
+        // from the first call on
+        const int batch = fx_batch(g->geom, nrhs);
+        tmnd_status st = tmnd_ensure_workspace(g, 2 * (size_t)fx_batch(g->geom, 1 << 30) * s32);
         if (st != TMND_OK) return st;
-        return apply_f32(g, (float2 *)out, (const float2 *)in, op & ~TMND_OP_F32, sigma, nrhs, (float2 *)g->work,
-                         (float2 *)((char *)g->work + s32), (cudaStream_t)stream);
+        return apply_f32(g, (float2 *)out, (const float2 *)in, op & ~TMND_OP_F32, sigma, nrhs, batch, (float2 *)g->work,
+                         (float2 *)((char *)g->work + batch * s32), (cudaStream_t)stream);
     }
     if (op & TMND_OP_S16) {
         TMND_ARG_CHECK(nrhs >= 1 && nrhs <= TMND_MAX_BATCH && out != in && ((uintptr_t)out & 15) == 0 &&

@@ -24,58 +24,9 @@
 #include <math.h>
 
 #include "hop_fx.cuh"
+#include "lattice.cuh"
 
 namespace {
-
-// n / d for n < 2^31 by a multiplication (Granlund and Montgomery, PLDI'94)
-struct FastDiv {
-    unsigned m;
-    int s, d;
-};
-FastDiv fast_div(int d) {
-    int s = 0;
-    while ((1ll << s) < d) s++;
-    return FastDiv{(unsigned)(((1ull << 32) * ((1ull << s) - (unsigned long long)d)) / (unsigned)d + 1), s, d};
-}
-__device__ __forceinline__ int fdiv(int n, const FastDiv &f) {
-    return (int)((__umulhi((unsigned)n, f.m) + (unsigned)n) >> f.s);
-}
-
-struct FxGeom {
-    int T, X, Y, Zh, Vh, Vs;  // Vs: V/2 rounded up to whole runs
-    int sx, st;               // half-index strides of x and t (y: Zh)
-    FastDiv dZh, dY, dX, dsx, dst;
-};
-FxGeom fx_geom(const Geom &g) {
-    const int sx = g.Zh * g.Y, st = sx * g.X;
-    return FxGeom{g.T, g.X, g.Y, g.Zh, g.Vh, (int)fx_sites(g.Vh), sx, st,
-                  fast_div(g.Zh), fast_div(g.Y), fast_div(g.X), fast_div(sx), fast_div(st)};
-}
-
-// Half-indices of the two neighbours in direction MU of site h of parity P.
-template <int MU, int P>
-__device__ __forceinline__ void neighbours(const FxGeom &g, int h, int &hf, int &hb) {
-    if (MU == 0) {
-        const int t = fdiv(h, g.dst);
-        hf = t + 1 == g.T ? h - (g.T - 1) * g.st : h + g.st;
-        hb = t == 0 ? h + (g.T - 1) * g.st : h - g.st;
-    } else if (MU == 1) {
-        const int q = fdiv(h, g.dsx), x = q - fdiv(q, g.dX) * g.X;
-        hf = x + 1 == g.X ? h - (g.X - 1) * g.sx : h + g.sx;
-        hb = x == 0 ? h + (g.X - 1) * g.sx : h - g.sx;
-    } else {
-        const int r = fdiv(h, g.dZh), q = fdiv(r, g.dY), y = r - q * g.Y;
-        if (MU == 2) {
-            hf = y + 1 == g.Y ? h - (g.Y - 1) * g.Zh : h + g.Zh;
-            hb = y == 0 ? h + (g.Y - 1) * g.Zh : h - g.Zh;
-        } else {
-            const int zh = h - r * g.Zh, t = fdiv(q, g.dX), x = q - t * g.X;
-            const bool odd = (P + t + x + y) & 1;  // z = 2 zh + odd
-            hf = !odd ? h : zh + 1 == g.Zh ? h - (g.Zh - 1) : h + 1;
-            hb = odd ? h : zh == 0 ? h + (g.Zh - 1) : h - 1;
-        }
-    }
-}
 
 // Spin projection of one flavour of a neighbour (in: its first word) for direction MU: digits of
 // chi = up -+ B lo, or of its complex conjugate for the backward hop (see hop_run).  G5IN: the input is
@@ -222,7 +173,7 @@ __device__ __forceinline__ int hop_sum(const FxShared &sm, int spin, long long v
 // takes direction mu, then adds up the four directions of spin mu: v 2^(e - 56), |v| <= 2^61.3, with the
 // flavour of the lane's half.  Returns e, the largest exponent among the neighbours.
 template <int P, bool G5IN>
-__device__ __forceinline__ int hop_run(const FxGeom &g, const int4 *__restrict__ links, const int4 *__restrict__ in,
+__device__ __forceinline__ int hop_run(const LatGeom &g, const int4 *__restrict__ links, const int4 *__restrict__ in,
                                        const int *__restrict__ ex, int h, FxShared &sm, long long v[3][2]) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int nb[2];
@@ -233,7 +184,7 @@ __device__ __forceinline__ int hop_run(const FxGeom &g, const int4 *__restrict__
         default: neighbours<3, P>(g, h, nb[0], nb[1]);
     }
     const int ef = __ldg(&ex[nb[0]]), eb = __ldg(&ex[nb[1]]), em = max(ef, eb);
-    const size_t mu_stride = 9 * (size_t)g.Vs;
+    const size_t mu_stride = 9 * fx_sites(g.Vh);
     const int4 *qf = in + fx_at(nb[0], 24), *qb = in + fx_at(nb[1], 24);
     const int4 *uf = links + ((size_t)P * 4 + w) * mu_stride + fx_at(h, 9);
     const int4 *ub = links + ((size_t)(1 - P) * 4 + w) * mu_stride + fx_at(nb[1], 9);
@@ -326,7 +277,7 @@ __device__ __forceinline__ void mac(int2 c, int h, int l, long long &x, long lon
 
 // even sites: t_e = kappa^2 A^-1 H psi  (DAG: kappa^2 A(-mu)^-1 H gamma_5 psi)
 template <bool DAG>
-__global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_even(FxGeom g, FxSite st, const int4 *__restrict__ links,
+__global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_even(LatGeom g, FxSite st, const int4 *__restrict__ links,
                                                                    FxIn psi, FxOut out, const int *__restrict__ done,
                                                                    int nrun, FxBatch bt) {
     __shared__ FxShared sm;
@@ -375,7 +326,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_even(FxGeom g, FxS
 
 // odd sites: y = A psi - H t  (DAG: A(-mu) psi - gamma_5 H t), then the epilogue.
 template <bool DAG, int EPI>
-__global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_odd(FxGeom g, FxSite st, const int4 *__restrict__ links,
+__global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_odd(LatGeom g, FxSite st, const int4 *__restrict__ links,
                                                                   FxIn psi, FxIn te, FxOdd ea, int nrun, FxBatch bt) {
     __shared__ FxShared sm;
     __shared__ double red[40];
@@ -690,7 +641,7 @@ void launch_fx_pack_links(const Geom &g, const double2 *canon, int4 *out, cudaSt
 void launch_fx_even(const Geom &g, const FxSite &st, const int4 *links, FxIn psi, FxOut out, bool dag,
                     const int *done, cudaStream_t s, const FxBatch &bt) {
     const FxGrid gr = fx_grid(g.Vh);
-    const FxGeom fg = fx_geom(g);
+    const LatGeom fg = lat_geom(g);
     if (dag)
         k_fx_even<true><<<dim3(gr.blocks, bt.nrhs), FX_THREADS, 0, s>>>(fg, st, links, psi, out, done, gr.runs, bt);
     else
@@ -700,7 +651,7 @@ void launch_fx_even(const Geom &g, const FxSite &st, const int4 *links, FxIn psi
 void launch_fx_odd(const Geom &g, const FxSite &st, const int4 *links, FxIn psi, FxIn te, bool dag, FxEpi epi,
                    FxOdd ea, cudaStream_t s, const FxBatch &bt) {
     const FxGrid gr = fx_grid(g.Vh);
-    const FxGeom fg = fx_geom(g);
+    const LatGeom fg = lat_geom(g);
     if (epi == FX_MMS_R) {
         ea.sig_e = exponent_of(ea.sigma);
         ea.sig = digits(ea.sigma, ea.sig_e);

@@ -83,7 +83,7 @@ int fx_batch(const Geom &g, int nrhs);
 constexpr int FX_RUN = 16;
 // first word of site h (component c at + c FX_RUN), for ncomp components per site
 __host__ __device__ inline int fx_at(int h, int ncomp) { return (h >> 4) * (ncomp * FX_RUN) + (h & 15); }
-inline size_t fx_sites(int Vh) { return ((size_t)Vh + 15) & ~(size_t)15; }
+__host__ __device__ inline size_t fx_sites(int Vh) { return ((size_t)Vh + 15) & ~(size_t)15; }
 inline size_t fx_link_words(int Vh) { return 2 * 4 * 9 * fx_sites(Vh); }
 inline size_t fx_bytes(int Vh) {
     return (fx_sites(Vh) * (NCOMP * sizeof(int4) + sizeof(int)) + 255) & ~(size_t)255;

@@ -22,114 +22,6 @@ tmnd_status launch_sap_color(const tmnd_gauge *g, const int bd[4], int color, do
 namespace {
 
 
-// Full-lattice doublet operator, output parity P, FP32:
-// y = (1 + i kp g5 t3 - kpp t1 [+ i s g5 t1 on odd sites]) x_P - kappa H x_{1-P}
-// nf = 2: doublet (24 components); nf = 1: one flavour, D_TM(+mu) (12 components, kpp and s ignored).
-__global__ void k_dnd_full(Geom g, double kappa, float kp, float kpp, float s_odd, const float2 *__restrict__ links,
-                           const float2 *__restrict__ in, float2 *__restrict__ out, int nf) {
-    const int ncomp = 12 * nf;
-    const int Vh = g.Vh;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * Vh; i += gridDim.x * blockDim.x) {
-        const int P = i / Vh, h = i % Vh, Q = 1 - P;
-        const int zh = h % g.Zh;
-        int r = h / g.Zh;
-        const int y0 = r % g.Y;
-        r /= g.Y;
-        const int x0 = r % g.X;
-        const int t0 = r / g.X;
-        const int z0 = 2 * zh + ((P + t0 + x0 + y0) & 1);
-        float2 acc[2][4][3];
-        for (int f = 0; f < 2; f++)
-            for (int s = 0; s < 4; s++)
-                for (int c = 0; c < 3; c++) acc[f][s][c] = make_float2(0.f, 0.f);
-        const int n[4] = {g.T, g.X, g.Y, g.Z};
-        for (int d = 0; d < 8; d++) {
-            const int mu = d >> 1;
-            const bool fwd = (d & 1) == 0;
-            int c[4] = {t0, x0, y0, z0};
-            float sg = 1.0f;
-            if (fwd) {
-                if (c[mu] + 1 == n[mu]) { c[mu] = 0; if (mu == 0 && g.apbc) sg = -1.0f; }
-                else c[mu]++;
-            } else {
-                if (c[mu] == 0) { c[mu] = n[mu] - 1; if (mu == 0 && g.apbc) sg = -1.0f; }
-                else c[mu]--;
-            }
-            const int hn = ((c[0] * g.X + c[1]) * g.Y + c[2]) * g.Zh + (c[3] >> 1);
-            const float2 *L = fwd ? links + ((size_t)(P * 4 + mu) * 9) * Vh : links + ((size_t)(Q * 4 + mu) * 9) * Vh;
-            const int hl = fwd ? h : hn;
-            float2 u[3][3];
-            for (int a = 0; a < 3; a++)
-                for (int b = 0; b < 3; b++) {
-                    const float2 w = fwd ? L[(size_t)(a * 3 + b) * Vh + hl] : L[(size_t)(b * 3 + a) * Vh + hl];
-                    u[a][b] = fwd ? w : make_float2(w.x, -w.y);
-                }
-            const float k = -(float)kappa * sg;
-            for (int f = 0; f < nf; f++) {
-                float2 ps[4][3];
-                for (int s = 0; s < 4; s++)
-                    for (int cc = 0; cc < 3; cc++) ps[s][cc] = in[((size_t)Q * ncomp + f * 12 + s * 3 + cc) * Vh + hn];
-                for (int cc = 0; cc < 3; cc++) {
-                    float2 gp[4];
-                    const float2 u0 = ps[0][cc], u1 = ps[1][cc], l0 = ps[2][cc], l1 = ps[3][cc];
-                    if (mu == 0) {
-                        gp[0] = make_float2(-l0.x, -l0.y); gp[1] = make_float2(-l1.x, -l1.y);
-                        gp[2] = make_float2(-u0.x, -u0.y); gp[3] = make_float2(-u1.x, -u1.y);
-                    } else if (mu == 1) {
-                        gp[0] = make_float2(l1.y, -l1.x); gp[1] = make_float2(l0.y, -l0.x);
-                        gp[2] = make_float2(-u1.y, u1.x); gp[3] = make_float2(-u0.y, u0.x);
-                    } else if (mu == 2) {
-                        gp[0] = make_float2(-l1.x, -l1.y); gp[1] = l0;
-                        gp[2] = u1; gp[3] = make_float2(-u0.x, -u0.y);
-                    } else {
-                        gp[0] = make_float2(l0.y, -l0.x); gp[1] = make_float2(-l1.y, l1.x);
-                        gp[2] = make_float2(-u0.y, u0.x); gp[3] = make_float2(u1.y, -u1.x);
-                    }
-                    const float sgn = fwd ? -1.0f : 1.0f;
-                    for (int s = 0; s < 4; s++)
-                        ps[s][cc] = make_float2(ps[s][cc].x + sgn * gp[s].x, ps[s][cc].y + sgn * gp[s].y);
-                }
-                for (int s = 0; s < 4; s++)
-                    for (int a = 0; a < 3; a++) {
-                        float2 v = make_float2(0.f, 0.f);
-                        for (int b = 0; b < 3; b++) v = cfma(u[a][b], ps[s][b], v);
-                        acc[f][s][a].x = fmaf(k, v.x, acc[f][s][a].x);
-                        acc[f][s][a].y = fmaf(k, v.y, acc[f][s][a].y);
-                    }
-            }
-        }
-        const float so = P == 1 ? s_odd : 0.0f;
-        if (nf == 1) {
-            for (int s = 0; s < 4; s++) {
-                const float g5 = s < 2 ? 1.0f : -1.0f;
-                for (int c = 0; c < 3; c++) {
-                    const float2 x0v = in[((size_t)P * 12 + s * 3 + c) * Vh + h];
-                    float2 o0;
-                    o0.x = x0v.x - kp * g5 * x0v.y + acc[0][s][c].x;
-                    o0.y = x0v.y + kp * g5 * x0v.x + acc[0][s][c].y;
-                    out[((size_t)P * 12 + s * 3 + c) * Vh + h] = o0;
-                }
-            }
-            continue;
-        }
-        for (int s = 0; s < 4; s++) {
-            const float g5 = s < 2 ? 1.0f : -1.0f;
-            for (int c = 0; c < 3; c++) {
-                const float2 x0v = in[((size_t)P * 24 + 0 * 12 + s * 3 + c) * Vh + h];
-                const float2 x1v = in[((size_t)P * 24 + 1 * 12 + s * 3 + c) * Vh + h];
-                // flavour 0: x0 + i kp g5 x0 - kpp x1 + i so g5 x1 ; flavour 1: x1 - i kp g5 x1 - kpp x0 + i so g5 x0
-                float2 o0, o1;
-                o0.x = x0v.x - kp * g5 * x0v.y - kpp * x1v.x - so * g5 * x1v.y + acc[0][s][c].x;
-                o0.y = x0v.y + kp * g5 * x0v.x - kpp * x1v.y + so * g5 * x1v.x + acc[0][s][c].y;
-                o1.x = x1v.x + kp * g5 * x1v.y - kpp * x0v.x - so * g5 * x0v.y + acc[1][s][c].x;
-                o1.y = x1v.y - kp * g5 * x1v.x - kpp * x0v.y + so * g5 * x0v.x + acc[1][s][c].y;
-                out[((size_t)P * 24 + 0 * 12 + s * 3 + c) * Vh + h] = o0;
-                out[((size_t)P * 24 + 1 * 12 + s * 3 + c) * Vh + h] = o1;
-            }
-        }
-    }
-}
-
 // complex dot <a, b> partials (double), n complex numbers
 __global__ void k_cdot(long n, const float2 *__restrict__ a, const float2 *__restrict__ b, double *part) {
     __shared__ double red[80];
@@ -232,8 +124,7 @@ struct MGSolver {
     float2 *cr, *ce, *cres, *cq[16], *cz[16];
 
     void apply(const float2 *in, float2 *out) {
-        k_dnd_full<<<nblk(n / 24), 256, 0, st>>>(g->geom, g->act.kappa, (float)g->st.kp, (float)g->st.kpp, (float)s,
-                                                g->links_f32, in, out, 2);
+        launch_dnd_full(g->geom, g->act.kappa, (float)g->st.kp, (float)g->st.kpp, (float)s, g->links_f32, in, out, 2, st);
     }
     // smoothing of D' x = r from x = 0: nu SAP sweeps (each: per colour the residual of the
     // whole lattice, then block-local MR on the blocks of that colour), or nu MR steps
@@ -408,9 +299,8 @@ extern "C" tmnd_status tmnd_mg_solve(tmnd_mg *mg, void *x, const void *b, double
 extern "C" tmnd_status tmnd_dnd_full_apply(tmnd_gauge *g, void *out, const void *in, double s, void *stream) {
     TMND_ARG_CHECK(g && out && in && out != in, "tmnd_dnd_full_apply: bad arguments");
     cudaGetLastError();
-    k_dnd_full<<<nblk(2L * g->geom.Vh), 256, 0, (cudaStream_t)stream>>>(
-        g->geom, g->act.kappa, (float)g->st.kp, (float)g->st.kpp, (float)s, g->links_f32, (const float2 *)in,
-        (float2 *)out, 2);
+    launch_dnd_full(g->geom, g->act.kappa, (float)g->st.kp, (float)g->st.kpp, (float)s, g->links_f32,
+                    (const float2 *)in, (float2 *)out, 2, (cudaStream_t)stream);
     TMND_CUDA_TRY(cudaGetLastError());
     return TMND_OK;
 }
@@ -436,8 +326,7 @@ extern "C" tmnd_status tmnd_mg_smooth_vectors(tmnd_gauge *g, void *vecs, int nve
     for (int v = 0; v < nvec; v++) {
         float2 *x = (float2 *)vecs + (size_t)v * n;
         for (int k = 0; k < iters; k++) {
-            k_dnd_full<<<nblk(2L * g->geom.Vh), 256, 0, st>>>(g->geom, g->act.kappa, (float)g->st.kp, 0.f, 0.f,
-                                                             g->links_f32, x, t, 1);
+            launch_dnd_full(g->geom, g->act.kappa, (float)g->st.kp, 0.f, 0.f, g->links_f32, x, t, 1, st);
             // r = -D x ; minimise |D (x + w r)| -> w = -(Dr... use the residual direction r = -Dx:
             // x <- x - w D x with w = <D x, x-ish>: plain MR on D x = 0: r = -D x, w = <D r, r>/<D r, D r>
             // (here r = -t and D r = -D t; the two signs cancel in w)

@@ -1027,8 +1027,8 @@ struct DCItem {
 // operator, r = d - (Qhat^2 + sigma) e (accurate to ~1e-7 of |d|, where the 16-bit
 // operator's own ~4e-5 would stall), and r is the next right-hand side.  A pair stops
 // once |r| <= target; the others go on, at most `max_inner` sloppy solves.
-tmnd_status apply_f32(tmnd_gauge *g, float2 *out, const float2 *in, int op, double sigma, int nrhs, float2 *te,
-                      float2 *yo, cudaStream_t s);
+tmnd_status apply_f32(tmnd_gauge *g, float2 *out, const float2 *in, int op, double sigma, int nrhs, int batch,
+                      float2 *te, float2 *yo, cudaStream_t s);
 
 // r = d - y (FP32) and block partials |r|^2 (FP64)
 __global__ void k_resid32(long n, const float2 *__restrict__ d, const float2 *__restrict__ y, float2 *__restrict__ r,
@@ -1124,7 +1124,7 @@ static tmnd_status inner_refine(tmnd_gauge *g, const MixedWork &mc, const InnerV
         for (int c = 0; c < R; c++) {
             if (!active[c]) continue;
             k_add32<<<nb, UPD_THREADS, 0, s>>>(n, mc.x32(c, 0), iv.e(c));
-            st = apply_f32(g, iv.yo + 0, iv.e(c), TMND_OP_QHAT2, sig[c], 1, iv.te, mc.x32(c, 0), s);
+            st = apply_f32(g, iv.yo + 0, iv.e(c), TMND_OP_QHAT2, sig[c], 1, 1, iv.te, mc.x32(c, 0), s);
             if (st != TMND_OK) return st;
             // apply_f32 left (Qhat^2 + sigma) e in iv.yo (its odd temporary is the slot's x32, free now)
             k_resid32<<<nb, UPD_THREADS, 0, s>>>(n, iv.d(c), iv.yo, mc.b32(c), part);

@@ -104,10 +104,6 @@ __device__ __forceinline__ float2 cfma_conj(float2 a, float2 b, float2 acc) {
 __device__ __forceinline__ float2 cmul_conj(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.x, b.y, -a.y * b.x));
 }
-__device__ __forceinline__ float2 cflip(float2 a, unsigned long long mask) {
-    const int m = mask ? (int)0x80000000 : 0;
-    return make_float2(__int_as_float(__float_as_int(a.x) ^ m), __int_as_float(__float_as_int(a.y) ^ m));
-}
 
 // Block-wide sum of one double (blockDim.x a multiple of 32, <= 1024); result valid in thread 0.
 __device__ __forceinline__ double block_sum(double v, double *smem /* >= 32 */) {
@@ -147,8 +143,6 @@ enum HopEpi {
     EPI_MMS_R = 3         // w = y + sigma * aux; r -= alpha w; partial |r|^2  (alpha from partials)
 };
 
-constexpr int HOP_THREADS = 128;
-
 struct HopEpiArgsF {
     float sigma;
     const float2 *aux;      // EPI_SHIFT: the vector multiplied by sigma
@@ -157,9 +151,14 @@ struct HopEpiArgsF {
 // The stencil in FP32 on FP32 planes with 18-real FP32 links (the FP32 operator:
 // accurate to ~1e-7, used for inner residuals of the defect correction)
 void launch_hop_even_f32(const Geom &g, const SiteTerm &st, const float2 *links, const float2 *psi_o, float2 *t_e,
-                         bool dag, cudaStream_t s);
+                         bool dag, int nrhs, cudaStream_t s);
 void launch_hop_odd_f32(const Geom &g, const SiteTerm &st, const float2 *links, const float2 *psi_o,
-                        const float2 *t_e, float2 *y_o, bool dag, HopEpi epi, const HopEpiArgsF &ea, cudaStream_t s);
+                        const float2 *t_e, float2 *y_o, bool dag, HopEpi epi, const HopEpiArgsF &ea, int nrhs,
+                        cudaStream_t s);
+// Full-lattice operator on FP32 vectors [parity][12 nf][V/2]: A x - kappa H x (+ i s gamma_5 tau_1 on odd
+// sites); nf = 2: doublet, nf = 1: one flavour, D_TM(+mu) (kpp and s ignored)
+void launch_dnd_full(const Geom &g, double kappa, float kp, float kpp, float s_odd, const float2 *links,
+                     const float2 *in, float2 *out, int nf, cudaStream_t s);
 
 // ------------------------------------------------- sloppy (16-bit) path
 
