@@ -19,7 +19,7 @@
 
 #include <vector>
 
-#include "tmnd_internal.cuh"
+#include "mg_transfer.cuh"
 
 struct tmnd_mg {
     tmnd_gauge *g;
@@ -532,20 +532,16 @@ extern "C" size_t tmnd_mg_coarse_bytes(const tmnd_mg *mg) {
 extern "C" tmnd_status tmnd_mg_restrict(const tmnd_mg *mg, void *out_c, const void *in_fine, int nrhs, void *stream) {
     TMND_ARG_CHECK(mg && out_c && in_fine && nrhs >= 1, "tmnd_mg_restrict: bad arguments");
     cudaGetLastError();
-    MGGeom m = mg_geom(mg);
-    k_mg_restrict<<<dim3(mg->nblock, nrhs), 256, 0, (cudaStream_t)stream>>>(m, mg->P, (const float2 *)in_fine, 24,
-                                                                           (float2 *)out_c, 0, 0);
-    TMND_CUDA_TRY(cudaGetLastError());
+    TMND_CUDA_TRY(launch_mg_restrict(mg->g->geom, mg->bd, mg->nbd, mg->nsb, mg->nv, mg->nblock, mg->P,
+                                     (const float2 *)in_fine, (float2 *)out_c, nrhs, (cudaStream_t)stream));
     return TMND_OK;
 }
 
 extern "C" tmnd_status tmnd_mg_prolong(const tmnd_mg *mg, void *out_fine, const void *in_c, int nrhs, void *stream) {
     TMND_ARG_CHECK(mg && out_fine && in_c && nrhs >= 1, "tmnd_mg_prolong: bad arguments");
     cudaGetLastError();
-    MGGeom m = mg_geom(mg);
-    k_mg_prolong<<<dim3(mg->nblock, nrhs), 256, 0, (cudaStream_t)stream>>>(m, mg->P, (const float2 *)in_c, 24,
-                                                                          (float2 *)out_fine, 0);
-    TMND_CUDA_TRY(cudaGetLastError());
+    TMND_CUDA_TRY(launch_mg_prolong(mg->g->geom, mg->bd, mg->nbd, mg->nsb, mg->nv, mg->nblock, mg->P,
+                                    (const float2 *)in_c, (float2 *)out_fine, nrhs, (cudaStream_t)stream));
     return TMND_OK;
 }
 
