@@ -178,10 +178,10 @@ tmnd_status s16_autotune(tmnd_gauge *g, int nrhs, cudaStream_t s, int *shape_out
     const size_t sb = spinor_bytes_prec(Vh, TMND_S16);
     const int maxgrid = hop_blocks_s16_max(g->geom);
     // scratch: in, t, y (16-bit) | partials [nrhs][2][grid] of the norms launch and [nrhs][grid]
-    // of the residual launch | (r, r) per RHS | residual planes in and out (FP32, nrhs each)
+    // of the residual launch | alpha per RHS | residual planes in and out (FP32, nrhs each)
     const size_t off_part = 3 * (size_t)nrhs * sb;
-    const size_t off_rr = (off_part + sizeof(double) * 3 * (size_t)nrhs * maxgrid + 255) & ~(size_t)255;
-    const size_t off_r = (off_rr + sizeof(double) * (size_t)nrhs + 255) & ~(size_t)255;
+    const size_t off_al = (off_part + sizeof(double) * 3 * (size_t)nrhs * maxgrid + 255) & ~(size_t)255;
+    const size_t off_r = (off_al + sizeof(double) * (size_t)nrhs + 255) & ~(size_t)255;
     const size_t r_elems = 24 * (size_t)Vh * nrhs;  // float2 per residual set
     const size_t total = off_r + 2 * sizeof(float2) * r_elems;
     char *buf = nullptr;
@@ -198,17 +198,17 @@ tmnd_status s16_autotune(tmnd_gauge *g, int nrhs, cudaStream_t s, int *shape_out
         return TMND_OK;
     }
     // biased 16-bit words of 0x4000 and unit scales: finite, data-independent timing; partials
-    // and residuals zero, (r, r) = the double of bytes 0x3f (a small positive number)
+    // and residuals zero, alpha = the double of bytes 0x3f (a small positive number)
     cudaMemsetAsync(buf, 0x40, off_part, s);
-    cudaMemsetAsync(buf + off_part, 0, off_rr - off_part, s);
-    cudaMemsetAsync(buf + off_rr, 0x3f, sizeof(double) * (size_t)nrhs, s);
+    cudaMemsetAsync(buf + off_part, 0, off_al - off_part, s);
+    cudaMemsetAsync(buf + off_al, 0x3f, sizeof(double) * (size_t)nrhs, s);
     cudaMemsetAsync(buf + off_r, 0, 2 * sizeof(float2) * r_elems, s);
     const S16In in = s16_in(buf, Vh);
     const S16Out te = s16_out(buf + (size_t)nrhs * sb, Vh), y = s16_out(buf + 2 * (size_t)nrhs * sb, Vh);
     const S16In tei{te.q, te.nrm}, yi{y.q, y.nrm};
     double *part = (double *)(buf + off_part);
     double *part_r = part + 2 * (size_t)nrhs * maxgrid;
-    const double *rr = (const double *)(buf + off_rr);
+    const double *alpha = (const double *)(buf + off_al);
     float2 *r_in = (float2 *)(buf + off_r), *r_out = r_in + r_elems;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
@@ -239,10 +239,8 @@ tmnd_status s16_autotune(tmnd_gauge *g, int nrhs, cudaStream_t s, int *shape_out
         e3a.r = r_out;
         e3a.r_stride = 24L * Vh;
         e3a.part_out = part_r;
-        e3a.part_in = part;
-        e3a.npart_in = hop_blocks_s16(g->geom, sh);
-        e3a.rr = rr;
-        e3a.rr_stride = 1;
+        e3a.alpha = alpha;
+        e3a.alpha_stride = 1;
         for (int obj = 0; obj < 2; obj++) {
             best[obj][sh] = 1e30f;
             for (int rep = 0; rep < 4 && err == cudaSuccess; rep++) {

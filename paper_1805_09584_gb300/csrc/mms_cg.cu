@@ -53,7 +53,7 @@ struct MMSState {
     double rr;          // (r, r) at the start of the current iteration
     double bb;          // (b, b)
     double alpha_old, beta_old;
-    double alpha;       // of the current iteration (FP64 path, k_alpha)
+    double alpha;       // of the current iteration (k_alpha)
     double zeta[NS], zeta_old[NS];
     int active[NS];
     int conv_iter[NS];
@@ -144,119 +144,126 @@ __device__ __forceinline__ MMSConst const_of(const MMSConst &c, const BatchConst
 
 // batched: block k initialises right-hand side k from partials [k][npart]
 __global__ void k_init_state_b(MMSState *st, size_t st_stride, const double *__restrict__ part, int npart,
-                               MMSConst c, BatchConst bc) {
+                               MMSConst c, BatchConst bc, int *done_all) {
     __shared__ double red[40];
     const MMSConst ck = const_of(c, bc, blockIdx.x);
-    init_state((MMSState *)((char *)st + blockIdx.x * st_stride), part + (size_t)blockIdx.x * npart, npart, ck, red);
+    st = (MMSState *)((char *)st + blockIdx.x * st_stride);
+    init_state(st, part + (size_t)blockIdx.x * npart, npart, ck, red);
+    if (threadIdx.x == 0 && st->done && atomicAdd(&done_all[1], 1) + 1 == (int)gridDim.x) done_all[0] = 1;
 }
 
-// Scalar step of the recursion (one block; thread 0 does the arithmetic).
-// j = position of this iteration inside its window.  part_norm: partials of |y|^2, |p|^2 (NULL: st->alpha
-// is already that of this iteration).
-__device__ void scalars_step(MMSState *st, MMSCoef *cf, const double *__restrict__ part_norm, int nb_hop,
-                             const double *__restrict__ part_rr, const MMSConst &c, int j, double *hist, int hist_cap,
-                             double *red) {
-    const int was_done = st->done;
-    double yy = 0, pp = 0, rr_new = 0;
-    if (!was_done) {
-        if (part_norm) {
-            yy = block_reduce_partials(part_norm, nb_hop, red);
-            pp = block_reduce_partials(part_norm + nb_hop, nb_hop, red);
-        }
-        rr_new = block_reduce_partials(part_rr, nb_hop, red);
-    }
-    if (threadIdx.x != 0) return;
-    if (j == 0) {  // a new window starts: x_i and p_i are up to date
-        for (int s = 0; s < c.nshift; s++) {
-            cf->P[s] = 1.0;
-            cf->a[s] = 0.0;
-            cf->touched[s] = 0;
-            for (int l = 0; l < WIN; l++) cf->Q[s][l] = cf->e[s][l] = 0.0;
-        }
+// Scalar step of the recursion (one block).  Every thread takes the base step; thread s then does shift s,
+// whose recursion needs nothing of the others (one thread for all shifts took 13-19 us per iteration with
+// 10-12 shifts, the eight of a window's coefficients included; now 4).  j = position of this iteration inside
+// its window.  st->alpha is already that of this iteration (k_alpha).  Returns true if the solve ended here.
+__device__ bool scalars_step(MMSState *st, MMSCoef *cf, int nb_hop, const double *__restrict__ part_rr,
+                             const MMSConst &c, int j, double *hist, int hist_cap, double *red) {
+    const int was_done = st->done, s = threadIdx.x;
+    const double rr_new = was_done ? 0.0 : block_reduce_partials(part_rr, nb_hop, red);
+    const bool mine = s < c.nshift;
+    if (j == 0 && mine) {  // a new window starts: x_i and p_i are up to date
+        cf->P[s] = 1.0;
+        cf->a[s] = 0.0;
+        cf->touched[s] = 0;
+        for (int l = 0; l < WIN; l++) cf->Q[s][l] = cf->e[s][l] = 0.0;
     }
     if (was_done) {
-        cf->skip = 1;
-        return;
+        if (s == 0) cf->skip = 1;
+        return false;
     }
-    const double alpha = part_norm ? st->rr / (yy + c.sigma0 * pp) : st->alpha;
-    const double beta = rr_new / st->rr;
-    if (!isfinite(alpha) || !isfinite(rr_new) || !isfinite(beta)) {
-        st->status = TMND_ERR_NAN;
-        st->done = 1;
-        cf->skip = 1;
-        return;
-    }
-    cf->skip = 0;
-    cf->beta = beta;
+    const double alpha = st->alpha, rr = st->rr, alpha_old = st->alpha_old, beta_old = st->beta_old, bb = st->bb;
+    const double beta = rr_new / rr;
     const int it = st->iter + 1;
-    if (hist && it <= hist_cap) {  // scalar history of the base recursion (Lanczos coefficients)
-        hist[2 * (it - 1)] = alpha;
-        hist[2 * (it - 1) + 1] = beta;
+    const bool bad = !isfinite(alpha) || !isfinite(rr_new) || !isfinite(beta);
+    __syncthreads();  // everyone has read the state
+    if (bad) {
+        if (s == 0) {
+            st->status = TMND_ERR_NAN;
+            st->done = 1;
+            cf->skip = 1;
+        }
+        return true;
     }
-    for (int s = 0; s < c.nshift; s++) {
-        if (!st->active[s]) continue;
+    if (mine && st->active[s]) {
         const double z = st->zeta[s], zo = st->zeta_old[s];
-        const double zn = z * zo * st->alpha_old /
-                          (alpha * st->beta_old * (zo - z) + zo * st->alpha_old * (1.0 + alpha * c.delta[s]));
+        const double zn = z * zo * alpha_old /
+                          (alpha * beta_old * (zo - z) + zo * alpha_old * (1.0 + alpha * c.delta[s]));
         const double ratio = zn / z;
         const double al = alpha * ratio;        // alpha_i
         const double be = beta * ratio * ratio; // beta_i
         // x_i += alpha_i p_i, with p_i = P p_i(k0) + sum_{l<j} Q_l r_l
-        cf->a[s] += al * cf->P[s];
+        const double P = cf->P[s];
+        cf->a[s] += al * P;
         for (int l = 0; l < j; l++) cf->e[s][l] += al * cf->Q[s][l];
         // p_i <- zeta_i' r' + beta_i p_i, r' in slot j
-        cf->P[s] *= be;
+        cf->P[s] = P * be;
         for (int l = 0; l < j; l++) cf->Q[s][l] *= be;
         cf->Q[s][j] = zn;
         cf->touched[s] = 1;
         st->zeta_old[s] = z;
         st->zeta[s] = zn;
-        if (s < c.nsolve && zn * zn * rr_new <= c.rho2 * st->bb) {
+        if (s < c.nsolve && zn * zn * rr_new <= c.rho2 * bb) {
             st->active[s] = 0;
             st->conv_iter[s] = it;
         }
     }
-    st->rr = rr_new;
-    st->alpha_old = alpha;
-    st->beta_old = beta;
-    st->iter = it;
-    if (!st->active[c.nsolve - 1] || it >= c.maxiter) st->done = 1;
+    __syncthreads();
+    const bool end = !st->active[c.nsolve - 1] || it >= c.maxiter;
+    if (s == 0) {
+        cf->skip = 0;
+        cf->beta = beta;
+        if (hist && it <= hist_cap) {  // scalar history of the base recursion (Lanczos coefficients)
+            hist[2 * (it - 1)] = alpha;
+            hist[2 * (it - 1) + 1] = beta;
+        }
+        st->rr = rr_new;
+        st->alpha_old = alpha;
+        st->beta_old = beta;
+        st->iter = it;
+        if (end) st->done = 1;
+    }
+    return end;
 }
 
-__global__ void k_scalars(MMSState *st, MMSCoef *cf, int nb_hop, const double *__restrict__ part_rr, MMSConst c, int j,
-                          double *hist, int hist_cap) {
+constexpr int SCAL_THREADS = 256;
+static_assert(SCAL_THREADS >= NS, "a thread per shift");
+
+__global__ void __launch_bounds__(SCAL_THREADS) k_scalars(MMSState *st, MMSCoef *cf, int nb_hop,
+                                                          const double *__restrict__ part_rr, MMSConst c, int j,
+                                                          double *hist, int hist_cap) {
     __shared__ double red[40];
-    scalars_step(st, cf, nullptr, nb_hop, part_rr, c, j, hist, hist_cap, red);
+    scalars_step(st, cf, nb_hop, part_rr, c, j, hist, hist_cap, red);
 }
 
-// alpha = (r, r) / (p, w), (p, w) = |Mhat p|^2 + sigma_0 |p|^2 from the partials of the first Mhat
-__global__ void k_alpha(MMSState *st, const double *__restrict__ part_norm, int nb_hop, double sigma0) {
-    __shared__ double red[40];
-    if (st->done) return;
-    const double yy = block_reduce_partials(part_norm, nb_hop, red);
-    const double pp = block_reduce_partials(part_norm + nb_hop, nb_hop, red);
-    if (threadIdx.x == 0) st->alpha = st->rr / (yy + sigma0 * pp);
-}
-
-// Batched: block k runs the scalar step of right-hand side k (state and
-// coefficients stride apart; partials [k][2][nb_hop] and [k][nb_hop]); the
-// scalar history is kept for k = 0.
-__global__ void k_scalars_b(MMSState *st, MMSCoef *cf, size_t st_stride, size_t cf_stride,
-                            const double *__restrict__ part_norm, int nb_hop, const double *__restrict__ part_rr,
-                            MMSConst c, BatchConst bc, int j, double *hist, int hist_cap) {
+// Batched: block k runs the scalar step of right-hand side k (state and coefficients stride apart; partials
+// [k][nb_hop]); the scalar history is kept for k = 0.  done_all[0] is set once all right-hand sides are done,
+// done_all[1] counts them.
+__global__ void __launch_bounds__(SCAL_THREADS) k_scalars_b(MMSState *st, MMSCoef *cf, size_t st_stride,
+                                                            size_t cf_stride, int nb_hop,
+                                                            const double *__restrict__ part_rr, MMSConst c,
+                                                            BatchConst bc, int j, double *hist, int hist_cap,
+                                                            int *done_all) {
     __shared__ double red[40];
     const int k = blockIdx.x;
     const MMSConst ck = const_of(c, bc, k);
-    scalars_step((MMSState *)((char *)st + k * st_stride), (MMSCoef *)((char *)cf + k * cf_stride),
-                 part_norm + (size_t)2 * k * nb_hop, nb_hop, part_rr + (size_t)k * nb_hop, ck, j,
-                 k == 0 ? hist : nullptr, hist_cap, red);
+    const bool end = scalars_step((MMSState *)((char *)st + k * st_stride), (MMSCoef *)((char *)cf + k * cf_stride),
+                                  nb_hop, part_rr + (size_t)k * nb_hop, ck, j, k == 0 ? hist : nullptr, hist_cap, red);
+    if (end && threadIdx.x == 0 && atomicAdd(&done_all[1], 1) + 1 == (int)gridDim.x) done_all[0] = 1;
 }
 
-// done_all = every right-hand side's solve is done
-__global__ void k_all_done(const MMSState *st, size_t st_stride, int nrhs, int *done_all) {
-    int d = 1;
-    for (int k = 0; k < nrhs; k++) d &= ((const MMSState *)((const char *)st + k * st_stride))->done;
-    *done_all = d;
+// alpha = (r, r) / (p, w), (p, w) = |Mhat p|^2 + sigma_0 |p|^2 from the partials [k][2][nb_hop] of the first
+// Mhat, block k for right-hand side k.  (When every block of the residual update worked alpha out for itself,
+// 16 right-hand sides cost each block 32 reductions, 20 us of a 54 us launch at 16^3x32.)
+__global__ void k_alpha(MMSState *st, size_t st_stride, const double *__restrict__ part_norm, int nb_hop, double sigma0,
+                        BatchConst bc) {
+    __shared__ double red[40];
+    const int k = blockIdx.x;
+    st = (MMSState *)((char *)st + k * st_stride);
+    if (st->done) return;
+    const double *part = part_norm + (size_t)2 * k * nb_hop;
+    const double yy = block_reduce_partials(part, nb_hop, red);
+    const double pp = block_reduce_partials(part + nb_hop, nb_hop, red);
+    if (threadIdx.x == 0) st->alpha = st->rr / (yy + (bc.on ? bc.sigma0[k] : sigma0) * pp);
 }
 
 // Windowed multi-shift update (end of each window): for every shift active
@@ -688,7 +695,7 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
         e1.done = &st->done;
         launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(p), te, false, &st->done, s);
         launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(p), fx_in(te), false, FX_STORE_NORMS, e1, s);
-        k_alpha<<<1, 256, 0, s>>>(st, part_norm, nb_hop, c.sigma0);
+        k_alpha<<<1, 256, 0, s>>>(st, 0, part_norm, nb_hop, c.sigma0, BatchConst());
         launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(y), te, true, &st->done, s);
         FxOdd e2 = {};
         e2.sigma = c.sigma0;
@@ -700,7 +707,7 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
         e2.done = &st->done;
         launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(y), fx_in(te), true, FX_MMS_R, e2, s);
         mark(1);
-        k_scalars<<<1, 256, 0, s>>>(st, cf, nb_hop, part_rr, c, j, hist, hist_cap);
+        k_scalars<<<1, SCAL_THREADS, 0, s>>>(st, cf, nb_hop, part_rr, c, j, hist, hist_cap);
         launch_fx_pupdate(g->geom, &cf->skip, &cf->beta, slot[j], p, s);
         if (j == WIN - 1) k_window<double2><<<nb_str, UPD_THREADS, 0, s>>>(n, cf, ring, ptrs, nshift);
         mark(2);
@@ -888,7 +895,7 @@ static tmnd_status mms_sloppy(tmnd_gauge *g, const MixedWork &m, const double *s
     const size_t cf_stride = (sizeof(MMSCoef) + 255) & ~(size_t)255;
     MMSState *st = (MMSState *)tail;
     MMSCoef *cf = (MMSCoef *)(tail + R * st_stride);
-    int *done_all = (int *)(tail + R * (st_stride + cf_stride));
+    int *done_all = (int *)(tail + R * (st_stride + cf_stride));  // flag, count
 
     MMSConst c = {};
     c.nshift = nshift;
@@ -917,8 +924,8 @@ static tmnd_status mms_sloppy(tmnd_gauge *g, const MixedWork &m, const double *s
     bt.shape = shape;
 
     k_init_s<<<dim3(nb_site, R), 128, 0, s>>>(Vh, v, part_str);
-    k_init_state_b<<<R, 256, 0, s>>>(st, st_stride, part_str, nb_site, c, bc);
-    k_all_done<<<1, 1, 0, s>>>(st, st_stride, R, done_all);
+    TMND_CUDA_TRY(cudaMemsetAsync(done_all, 0, 2 * sizeof(int), s));
+    k_init_state_b<<<R, 256, 0, s>>>(st, st_stride, part_str, nb_site, c, bc, done_all);
     TMND_CUDA_TRY(cudaGetLastError());
 
     auto body = [&](int k, auto mark) {
@@ -929,6 +936,7 @@ static tmnd_status mms_sloppy(tmnd_gauge *g, const MixedWork &m, const double *s
         e1.done = done_all;
         launch_hop_even_s16(g->geom, g->stf, g->links_s16, p16i, te16, false, done_all, s, bt);
         launch_hop_odd_s16(g->geom, g->stf, g->links_s16, p16i, te16i, y16, false, EPI_STORE_NORMS, e1, s, bt);
+        k_alpha<<<R, 256, 0, s>>>(st, st_stride, part_norm, nb_hop, c.sigma0, bc);
         launch_hop_even_s16(g->geom, g->stf, g->links_s16, y16i, te16, true, done_all, s, bt);
         S16EpiArgs e2 = {};
         e2.sigma = c.sigma0;
@@ -937,18 +945,15 @@ static tmnd_status mms_sloppy(tmnd_gauge *g, const MixedWork &m, const double *s
         e2.r = m.ring(0, j);
         e2.r_stride = (long)WIN * n;
         e2.part_out = part_rr;
-        e2.part_in = part_norm;
-        e2.npart_in = nb_hop;
-        e2.rr = &st->rr;
-        e2.rr_stride = (int)(st_stride / sizeof(double));
+        e2.alpha = &st->alpha;
+        e2.alpha_stride = (int)(st_stride / sizeof(double));
         e2.done = done_all;
         e2.per_rhs_sigma = bc.on;
         for (int q = 0; q < R && bc.on; q++) e2.sigma_k[q] = bc.sigma0[q];
         launch_hop_odd_s16(g->geom, g->stf, g->links_s16, y16i, te16i, S16Out{}, true, EPI_MMS_R, e2, s, bt);
         mark(1);
-        k_scalars_b<<<R, 256, 0, s>>>(st, cf, st_stride, cf_stride, part_norm, nb_hop, part_rr, c, bc, j, hist,
-                                      hist_cap);
-        k_all_done<<<1, 1, 0, s>>>(st, st_stride, R, done_all);
+        k_scalars_b<<<R, SCAL_THREADS, 0, s>>>(st, cf, st_stride, cf_stride, nb_hop, part_rr, c, bc, j, hist, hist_cap,
+                                               done_all);
         k_pupdate_s<<<dim3(nb_site, R), 128, 0, s>>>(Vh, cf, cf_stride, v, j);
         if (j == WIN - 1) k_window_s<<<dim3(nb_str, R), UPD_THREADS, 0, s>>>(cf, cf_stride, v);
         mark(2);

@@ -187,12 +187,7 @@ __global__ void __launch_bounds__(NT, MB) k_hop_odd_s16(Geom g, SiteTermF st, co
     const int Vh = g.Vh;
     constexpr bool SUMS = EPI == EPI_STORE_NORMS || EPI == EPI_MMS_R;
     if (EPI == EPI_MMS_R) {
-        for (int k = 0; k < bt.nrhs; k++) {
-            const double yy = block_reduce_partials(ea.part_in + (size_t)(2 * k) * ea.npart_in, ea.npart_in, red);
-            const double pp = block_reduce_partials(ea.part_in + (size_t)(2 * k + 1) * ea.npart_in, ea.npart_in, red);
-            const double sg = ea.per_rhs_sigma ? ea.sigma_k[k] : ea.sigma;
-            if (threadIdx.x == 0) alpha_s[k] = (float)(ea.rr[(size_t)k * ea.rr_stride] / (yy + sg * pp));
-        }
+        if (threadIdx.x < bt.nrhs) alpha_s[threadIdx.x] = (float)ea.alpha[(size_t)threadIdx.x * ea.alpha_stride];
     }
     if (SUMS)
         for (int k = 0; k < 2 * bt.nrhs; k++) part[k * blockDim.x + threadIdx.x] = 0.0;

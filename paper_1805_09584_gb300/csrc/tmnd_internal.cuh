@@ -140,7 +140,7 @@ enum HopEpi {
     EPI_STORE = 0,        // out = y
     EPI_STORE_NORMS = 1,  // out = y; partials |y|^2, |in|^2
     EPI_SHIFT = 2,        // out = y + sigma * aux
-    EPI_MMS_R = 3         // w = y + sigma * aux; r -= alpha w; partial |r|^2  (alpha from partials)
+    EPI_MMS_R = 3         // w = y + sigma * aux; r -= alpha w; partial |r|^2
 };
 
 struct HopEpiArgsF {
@@ -203,12 +203,10 @@ struct S16EpiArgs {
     float2 *r;              // EPI_MMS_R: updated residual (FP32 planes, written)
     const float2 *r_in;     // EPI_MMS_R: residual before the update
     double *part_out;       // block partials: EPI_STORE_NORMS [rhs][2][grid], EPI_MMS_R [rhs][grid]
-    const double *part_in;  // EPI_MMS_R: the previous launch's [rhs][2][npart_in]
-    int npart_in;
-    const double *rr;       // EPI_MMS_R: (r, r) of right-hand side k at rr[k * rr_stride]
+    const double *alpha;    // EPI_MMS_R: step length of right-hand side k at alpha[k * alpha_stride]
     const int *done;
     long r_stride;          // EPI_MMS_R: float2 elements between right-hand sides of r / r_in
-    int rr_stride;          // doubles between right-hand sides of rr
+    int alpha_stride;       // doubles between right-hand sides of alpha
 };
 
 // Several right-hand sides in one stencil launch (links read once, shared in cache):
