@@ -185,11 +185,11 @@ tmnd_status tm_nd_apply_noalloc(const tmnd_gauge *g, void *out, const void *in, 
 
 /* Launch-shape autotuner of the sloppy (16-bit) stencil.  Its kernels run in
  * TMND_S16_SHAPES launch variants: 4 compiled shapes (threads per block x resident blocks
- * per SM the register budget is cut for x next-direction prefetch) x 4 loop orders (0: every
- * block walks its own chunk of sites, all right-hand sides of a site in turn; 1: the chunk
+ * per SM the register budget is cut for x next-direction prefetch; shape 0 takes one right-hand
+ * side per pass over a block's tile of sites, the others two) x 4 loop orders (0: every
+ * block walks its own tiles, all right-hand sides of a tile in turn; 1: its tiles
  * once per right-hand side; 2: all blocks sweep the lattice together by grid stride, all
- * right-hand sides of a site in turn; 3: grid stride over (group of 32 sites, right-hand
- * side) items, one per warp, a group's right-hand sides on consecutive warps);
+ * right-hand sides of a tile in turn; 3: grid stride over (tile, right-hand side) items);
  * tmnd_s16_shape_info.  For each lattice and number of right-hand sides per launch (1..16)
  * the library times every variant once on the current device, on scratch data, CUDA events,
  * best of 3 after a warm-up, for two sequences of 4 launches: (a) one 16-bit Qhat^2 + sigma

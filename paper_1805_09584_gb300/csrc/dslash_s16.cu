@@ -7,7 +7,7 @@
 
 #include "s16_kernels.cuh"
 
-#define TMND_S16_DECL(I, T, B, P)                                                                               \
+#define TMND_S16_DECL(I, T, B, P, R)                                                                               \
     int s16_per_sm_##I();                                                                                       \
     void s16_even_##I(const Geom &g, const SiteTermF &st, const int2 *links, S16In in, S16Out out, bool dag,   \
                       const int *done, cudaStream_t s, const S16Batch &bt, int nb);                             \
@@ -19,19 +19,18 @@ TMND_S16_SHAPE_LIST(TMND_S16_DECL)
 namespace {
 
 struct ShapeDesc {
-    int threads, minb, pf;
+    int threads, minb, pf, rp;
 };
 constexpr ShapeDesc kShapes[] = {
-#define TMND_S16_DESC(I, T, B, P) {T, B, P},
+#define TMND_S16_DESC(I, T, B, P, R) {T, B, P, R},
     TMND_S16_SHAPE_LIST(TMND_S16_DESC)
 #undef TMND_S16_DESC
 };
 constexpr int NCOMPILED = sizeof(kShapes) / sizeof(kShapes[0]);
 // a launch variant = compiled shape (v % NCOMPILED) x loop order (v / NCOMPILED): 0 = every
-// block walks its own chunk of sites, all right-hand sides of a site in turn; 1 = the same
-// chunk once per right-hand side; 2 = all blocks sweep the lattice together (grid stride),
-// all right-hand sides of a site in turn; 3 = grid stride over (32-site group, right-hand
-// side) items, one per warp
+// block walks its own tiles of sites, all right-hand sides of a tile in turn; 1 = the same
+// tiles once per right-hand side; 2 = all blocks sweep the lattice together (grid stride),
+// all right-hand sides of a tile in turn; 3 = grid stride over (tile, right-hand side) items
 constexpr int NORDERS = 4;
 constexpr int NSHAPES = NORDERS * NCOMPILED;
 static_assert(NSHAPES == TMND_S16_SHAPES, "variant count of include/tmnd.h");
@@ -46,7 +45,7 @@ int per_sm(int shape) {
     if (dev < 0 || dev >= 64) dev = 0;
     if (!g_per_sm[dev][shape]) {
         switch (shape) {
-#define TMND_S16_OCC(I, T, B, P) \
+#define TMND_S16_OCC(I, T, B, P, R) \
     case I: g_per_sm[dev][I] = s16_per_sm_##I(); break;
             TMND_S16_SHAPE_LIST(TMND_S16_OCC)
 #undef TMND_S16_OCC
@@ -86,12 +85,13 @@ std::array<int, 6> tune_key(const Geom &g, int nrhs) {
 }  // namespace
 
 // blocks of a stencil launch in this shape: one per resident slot on every SM (persistent
-// grid), at most one site per thread
+// grid), at most one per tile
 int hop_blocks_s16(const Geom &g, int shape) {
     if (shape < 0 || shape >= NSHAPES) shape = 0;
-    const int nt = kShapes[shape % NCOMPILED].threads;
+    const ShapeDesc &d = kShapes[shape % NCOMPILED];
+    const int sites = d.threads / (2 * d.rp);  // per tile
     const int cap = sm_count() * per_sm(shape);
-    const int want = (g.Vh + nt - 1) / nt;
+    const int want = (g.Vh + sites - 1) / sites;
     return want < cap ? want : cap;
 }
 
@@ -122,7 +122,7 @@ void launch_hop_even_s16(const Geom &g, const SiteTermF &st, const int2 *links, 
     bt.order = shape / NCOMPILED;
     const int nb = hop_blocks_s16(g, shape);
     switch (shape % NCOMPILED) {
-#define TMND_S16_EVEN(I, T, B, P) \
+#define TMND_S16_EVEN(I, T, B, P, R) \
     case I: s16_even_##I(g, st, links, in, out, dag, done, s, bt, nb); break;
         TMND_S16_SHAPE_LIST(TMND_S16_EVEN)
 #undef TMND_S16_EVEN
@@ -138,7 +138,7 @@ void launch_hop_odd_s16(const Geom &g, const SiteTermF &st, const int2 *links, S
     bt.order = shape / NCOMPILED;
     const int nb = hop_blocks_s16(g, shape);
     switch (shape % NCOMPILED) {
-#define TMND_S16_ODD(I, T, B, P) \
+#define TMND_S16_ODD(I, T, B, P, R) \
     case I: s16_odd_##I(g, st, links, psi, te, out, dag, epi, ea, s, bt, nb); break;
         TMND_S16_SHAPE_LIST(TMND_S16_ODD)
 #undef TMND_S16_ODD

@@ -15,277 +15,317 @@
 //     conj(row0 x row1) (det U = +1, Sec. 2: U in SU(3)).  The antiperiodic
 //     sign is applied in the kernel, never folded into links.
 //
-// The kernels read every neighbour word straight from global memory; the
-// arithmetic is in s16_hop.cuh.
-//   * PF: the words of the next direction are loaded before the current one is
-//     processed (more memory requests in flight per warp).
-//   * Links are read once per launch, so their loads bypass L1.
+// A block works on tiles of consecutive sites, a thread per site, flavour and one of RP right-hand sides:
+// lane bit 4 is the flavour, for RP = 2 bit 3 the right-hand side, the low bits the site.  The tile's eight
+// links per site are decoded once, row 2 included, into shared memory as FP32 and serve both flavours and
+// every right-hand side; the neighbours' words come straight from global memory (PF: those of the next
+// direction are loaded before the current one is processed).  Arithmetic in s16_hop.cuh.
+// RP = 2 halves the shared-memory traffic for the links (a warp's 16-byte reads fall on 8 sites, one line,
+// instead of 16; with RP = 1 that traffic keeps the L1 data pipe 68 % busy): 7 % faster at 16^3x32 with 8 right-hand
+// sides, 2 % slower at 24^3x48, useless for one.
+//
+// The form before this one had one thread per site for both flavours, which decoded and rebuilt the links
+// for every right-hand side (60 of 225 instructions per direction) at 168 registers, 12 warps per SM, and was
+// bound by issue and latency together.  Four launches of Qhat^2 + sigma, before and now: 24^3x48 1 right-hand
+// side 0.22 -> 0.23 ms, 8 1.47 -> 1.29 ms; 16^3x32 8 0.39 -> 0.29 ms; an iteration of the multi-shift solver at
+// 24^3x48 with 8 (the residual update's FP32 planes loaded all at once) 1.9 -> 1.33 ms.  Now: FP32 pipe 53 %,
+// issue 55 %, 17 warps per SM.
 //
 // This header holds the kernel templates; each compiled launch shape is instantiated
 // in a translation unit of its own (dslash_s16_v*.cu, built in parallel) through
 // TMND_S16_DEFINE_SHAPE; dslash_s16.cu dispatches between them and runs the autotuner.
 #pragma once
 
+#include "lattice.cuh"
 #include "s16_hop.cuh"
 
 namespace {
 
+// Launch shapes the kernels are compiled in: threads per block, resident blocks per SM the register budget is
+// cut for, next-direction prefetch, right-hand sides per pass.  The autotuner times each on the GPU per
+// (lattice, right-hand sides per launch) and keeps the fastest; shape 0 is the default.
+#define TMND_S16_SHAPE_LIST(X) X(0, 128, 4, true, 1) X(1, 128, 5, true, 2) X(2, 64, 8, true, 2) X(3, 64, 10, true, 2)
 
-// Launch shapes the kernels are compiled in: threads per block, resident blocks per
-// SM the register budget is cut for, next-direction prefetch.  The autotuner below
-// times each on the GPU per (lattice, right-hand sides per launch) and keeps the
-// fastest; shape 0 is the default (168 registers, 12 warps per SM; 4 blocks of 128
-// at 128 registers spill and ran slower).
-#define TMND_S16_SHAPE_LIST(X) X(0, 128, 3, true) X(1, 128, 3, false) X(2, 64, 6, true) X(3, 256, 1, true)
-
-__device__ __forceinline__ int2 ld_link(const int2 *p) {
-    int2 r;
-    asm("ld.global.nc.L1::no_allocate.v2.s32 {%0, %1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(p));
-    return r;
-}
-
-__device__ __forceinline__ void load_raw(const int4 *__restrict__ q, const float *__restrict__ nrm, int Vh, int hn,
-                                         const int2 *__restrict__ L, int hl, Raw &r) {
-#pragma unroll
-    for (int f = 0; f < 2; f++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) r.q[f][j] = __ldg(&q[s16_qi(f * 3 + j, hn)]);
-#pragma unroll
-    for (int j = 0; j < 3; j++) r.l[j] = ld_link(&L[s16_li(j, hl)]);
-    r.nrm = __ldg(&nrm[s16_ni(hn)]);
-}
-
-// neighbour table of one site: direction d = 2 mu + (0 forward, 1 backward)
-struct Nbr {
-    int hn[8], hl[8];
-    float sg[8];
+template <int NT, int RP>
+struct Tile {
+    static constexpr int SITES = NT / (2 * RP);
+    LinkTile<SITES> links;
+    int nb[8][SITES];  // neighbours, direction 2 mu + (0 forward, 1 backward)
 };
 
-template <int P>
-__device__ __forceinline__ void neighbours(const Geom &g, int h, Nbr &n) {
-    int zh = h % g.Zh;
-    int r = h / g.Zh;
-    const int y = r % g.Y;
-    r /= g.Y;
-    const int x = r % g.X;
-    const int t = r / g.X;
-    const int z = 2 * zh + ((P + t + x + y) & 1);
-    auto idx = [&](int tt, int xx, int yy, int zz) { return ((tt * g.X + xx) * g.Y + yy) * g.Zh + (zz >> 1); };
-    const int tf = (t + 1 == g.T) ? 0 : t + 1, tb = (t == 0) ? g.T - 1 : t - 1;
-    const int xf = (x + 1 == g.X) ? 0 : x + 1, xb = (x == 0) ? g.X - 1 : x - 1;
-    const int yf = (y + 1 == g.Y) ? 0 : y + 1, yb = (y == 0) ? g.Y - 1 : y - 1;
-    const int zf = (z + 1 == g.Z) ? 0 : z + 1, zb = (z == 0) ? g.Z - 1 : z - 1;
-    n.hn[0] = idx(tf, x, y, z); n.hn[1] = idx(tb, x, y, z);
-    n.hn[2] = idx(t, xf, y, z); n.hn[3] = idx(t, xb, y, z);
-    n.hn[4] = idx(t, x, yf, z); n.hn[5] = idx(t, x, yb, z);
-    n.hn[6] = idx(t, x, y, zf); n.hn[7] = idx(t, x, y, zb);
+// Neighbours and decoded links of the tile that starts at site h0 (output parity P); links of direction d:
+// forward from this parity's sites, backward from the other's.
+template <int P, int NT, int RP>
+__device__ __forceinline__ void load_tile(const LatGeom &g, int apbc, const int2 *__restrict__ links, int h0,
+                                          Tile<NT, RP> &t) {
+    constexpr int SITES = Tile<NT, RP>::SITES;
+    const size_t stride = 3 * (size_t)g.Vh;
+    const int2 *Lp = links + (size_t)P * 4 * stride, *Lq = links + (size_t)(1 - P) * 4 * stride;
 #pragma unroll
-    for (int d = 0; d < 8; d++) {
-        n.hl[d] = (d & 1) ? n.hn[d] : h;  // forward: link at x; backward: link at x - mu
-        n.sg[d] = 1.0f;
+    for (int w = 0; w < 2 / RP; w++) {
+        const int item = threadIdx.x + w * NT, i = item % SITES, mu = item / SITES, h = min(h0 + i, g.Vh - 1);
+        int hf, hb;
+        float sf = 1.0f, sb = 1.0f;
+        if (mu == 0) {
+            neighbours<0, P>(g, h, hf, hb);
+            if (apbc) {  // a hop across the time boundary carries -1
+                sf = hf < h ? -1.0f : 1.0f;
+                sb = hb > h ? -1.0f : 1.0f;
+            }
+        } else if (mu == 1) {
+            neighbours<1, P>(g, h, hf, hb);
+        } else if (mu == 2) {
+            neighbours<2, P>(g, h, hf, hb);
+        } else {
+            neighbours<3, P>(g, h, hf, hb);
+        }
+        t.nb[2 * mu][i] = hf;
+        t.nb[2 * mu + 1][i] = hb;
+        f2 u[9];
+        decode_link(Lp + mu * stride, h, sf, u);
+        t.links.put(2 * mu, i, u);
+        decode_link(Lq + mu * stride, hb, sb, u);
+        t.links.put(2 * mu + 1, i, u);
     }
-    if (g.apbc && t + 1 == g.T) n.sg[0] = -1.0f;
-    if (g.apbc && t == 0) n.sg[1] = -1.0f;
 }
 
-// links of direction d: forward from this parity's planes, backward from the other's
-template <int P, int D>
-__device__ __forceinline__ const int2 *link_base(const int2 *__restrict__ links, int Vh) {
-    constexpr int par = (D & 1) ? 1 - P : P;
-    return links + ((size_t)par * 4 + D / 2) * 3 * Vh;
-}
-
-template <int P, int D, bool G5IN, bool PF>
-__device__ __forceinline__ void hop_seq(const int2 *__restrict__ links, const int4 *__restrict__ q,
-                                        const float *__restrict__ nrm, int Vh, const Nbr &n, const Raw &cur,
-                                        f2 acc[4][3][2]) {
+template <int D, bool G5IN, bool PF, int NT, int RP>
+__device__ __forceinline__ void hop_seq(const Tile<NT, RP> &t, int i, const S16In &in, int f, const Raw &cur, f2 up[3][2],
+                                        f2 lo[3][2]) {
     Raw nxt;
-    if constexpr (PF && D < 7) load_raw(q, nrm, Vh, n.hn[D + 1], link_base<P, D + 1>(links, Vh), n.hl[D + 1], nxt);
-    hop_dir<D / 2, (D & 1) ? -1 : 1, G5IN, D == 0>(cur, n.sg[D], acc);
+    if constexpr (PF && D < 7) load_raw(in, f, t.nb[D + 1][i], nxt);
+    f2 u[9];
+    t.links.get(D, i, u);
+    hop_dir<D / 2, (D & 1) ? -1 : 1, G5IN, D == 0>(cur, u, up, lo);
     if constexpr (D < 7) {
-        if constexpr (!PF) load_raw(q, nrm, Vh, n.hn[D + 1], link_base<P, D + 1>(links, Vh), n.hl[D + 1], nxt);
-        hop_seq<P, D + 1, G5IN, PF>(links, q, nrm, Vh, n, nxt, acc);
+        if constexpr (!PF) load_raw(in, f, t.nb[D + 1][i], nxt);
+        hop_seq<D + 1, G5IN, PF, NT, RP>(t, i, in, f, nxt, up, lo);
+    }
+}
+// H psi at tile site i, flavour f: v[spin*3 + colour]
+template <bool G5IN, bool PF, int NT, int RP>
+__device__ __forceinline__ void hop_all(const Tile<NT, RP> &t, int i, const S16In &in, int f, f2 v[12]) {
+    f2 up[3][2], lo[3][2];
+    Raw r;
+    load_raw(in, f, t.nb[0][i], r);
+    hop_seq<0, G5IN, PF, NT, RP>(t, i, in, f, r, up, lo);
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        v[c] = make_float2(up[c][0].x, up[c][1].x);
+        v[3 + c] = make_float2(up[c][0].y, up[c][1].y);
+        v[6 + c] = make_float2(lo[c][0].x, lo[c][1].x);
+        v[9 + c] = make_float2(lo[c][0].y, lo[c][1].y);
     }
 }
 
-template <int P, bool G5IN, bool PF>
-__device__ __forceinline__ void hop_all(const Geom &g, const int2 *__restrict__ links, const int4 *__restrict__ q,
-                                        const float *__restrict__ nrm, int h, f2 acc[4][3][2]) {
-    Nbr n;
-    neighbours<P>(g, h, n);
-    Raw r0;
-    load_raw(q, nrm, g.Vh, n.hn[0], link_base<P, 0>(links, g.Vh), n.hl[0], r0);
-    hop_seq<P, 0, G5IN, PF>(links, q, nrm, g.Vh, n, r0, acc);
-}
-
-// Loop order 3: grid stride over (group of 32 consecutive sites, right-hand side) work items,
-// one per warp, the right-hand sides of a group on consecutive warps.  All warps move through
-// the lattice together as in order 2, but each carries one right-hand side, so the band of
-// sites in flight (and the neighbour words it keeps live in L2) is nrhs times narrower; the
-// warps of a group read the same links side by side.
-template <class F>
-__device__ __forceinline__ void grid_stride_rhs_warps(int Vh, const S16Batch &bt, F &&site) {
-    const int lane = threadIdx.x & 31;
-    const long nwarps = (long)gridDim.x * (blockDim.x >> 5);
-    const long items = (long)((Vh + 31) >> 5) * bt.nrhs;
-    for (long w = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < items; w += nwarps) {
-        const int k = (int)(w % bt.nrhs);
-        const int h = (int)(w / bt.nrhs) * 32 + lane;
-        if (h >= Vh || (bt.rdone && bt.rdone[k * bt.rdone_stride])) continue;
-        site(h, k);
+// The loop orders over tiles and right-hand sides.  tile(w) prepares a tile (all threads), site(k) does right-hand
+// sides k .. k + RP - 1 of it.
+template <int RP, class F, class G>
+__device__ __forceinline__ void walk(int ntile, const S16Batch &bt, F &&tile, G &&site) {
+    const int t0 = (int)((long long)ntile * blockIdx.x / gridDim.x), t1 = (int)((long long)ntile * (blockIdx.x + 1) / gridDim.x);
+    auto off = [&](int k) {  // nothing left to do in this group
+        bool o = bt.rdone != nullptr;
+        for (int q = k; q < k + RP && q < bt.nrhs && o; q++) o = bt.rdone[q * bt.rdone_stride];
+        return o;
+    };
+    const int groups = (bt.nrhs + RP - 1) / RP;
+    if (bt.order == 3) {  // grid stride over (tile, right-hand sides) items
+        const long items = (long)ntile * groups;
+        for (long w = blockIdx.x; w < items; w += gridDim.x) {
+            const int k = (int)(w % groups) * RP;
+            if (off(k)) continue;
+            tile((int)(w / groups));
+            site(k);
+        }
+    } else if (bt.order == 2) {  // grid stride over tiles: all blocks move through the lattice together, so every
+                                 // right-hand side's neighbours stay in L2 while the band passes
+        for (int w = blockIdx.x; w < ntile; w += gridDim.x) {
+            tile(w);
+            for (int k = 0; k < bt.nrhs; k += RP)
+                if (!off(k)) site(k);
+        }
+    } else if (bt.order == 1) {  // each group of right-hand sides over the block's own tiles, one after another
+        for (int k = 0; k < bt.nrhs; k += RP)
+            for (int w = t0; w < t1 && !off(k); w++) {
+                tile(w);
+                site(k);
+            }
+    } else {  // the block's own tiles, every right-hand side of a tile before the next
+        for (int w = t0; w < t1; w++) {
+            tile(w);
+            for (int k = 0; k < bt.nrhs; k += RP)
+                if (!off(k)) site(k);
+        }
     }
 }
 
-template <bool DAG, bool PF, int NT, int MB>
-__global__ void __launch_bounds__(NT, MB) k_hop_even_s16(Geom g, SiteTermF st, const int2 *__restrict__ links,
-                                                         S16In in, S16Out out, const int *__restrict__ done,
-                                                         int chunk, S16Batch bt) {
+// A thread's place: flavour, site of the tile, right-hand side of the pass
+template <int RP>
+struct Place {
+    int f, i, q;
+    __device__ __forceinline__ Place() {
+        const int lane = threadIdx.x & 31;
+        f = lane >> 4;
+        i = (threadIdx.x >> 5) * (16 / RP) + (lane & (16 / RP - 1));
+        q = RP == 2 ? lane >> 3 & 1 : 0;
+    }
+    // this thread's right-hand side of the pass from k on; on = false (and another's number) if it has nothing to do
+    __device__ __forceinline__ int rhs(int k, const S16Batch &bt, bool &on) const {
+        if (RP == 1) return k;
+        const bool mine = k + q < bt.nrhs && !(bt.rdone && bt.rdone[(k + q) * bt.rdone_stride]);
+        on = on && mine;
+        return k + q < bt.nrhs ? k + q : k;
+    }
+};
+
+template <bool DAG, bool PF, int NT, int MB, int RP>
+__global__ void __launch_bounds__(NT, MB) k_hop_even_s16(LatGeom g, int apbc, SiteTermF st, const int2 *__restrict__ links,
+                                                         S16In in, S16Out out, const int *__restrict__ done, int ntile,
+                                                         S16Batch bt) {
+    __shared__ Tile<NT, RP> t;
     if (done && *done) return;
-    const int h_end = min(g.Vh, (int)(blockIdx.x + 1) * chunk);
-    auto site = [&](int h, int k) {
-        const S16In ik = s16_at(in, k * bt.stride);
-        f2 acc[4][3][2];
-        hop_all<0, DAG, PF>(g, links, ik.q, ik.nrm, h, acc);
-        f2 o[4][3][2];
-        even_term<DAG>(st, acc, o);
-        const S16Out ok = s16_at(out, k * bt.stride);
-        store_site(ok.q, ok.nrm, g.Vh, h, o);
+    const Place<RP> pl;
+    const int f = pl.f;
+    int h = 0;
+    auto tile = [&](int w) {
+        __syncthreads();  // the previous tile is done with
+        load_tile<0, NT, RP>(g, apbc, links, w * Tile<NT, RP>::SITES, t);
+        h = w * Tile<NT, RP>::SITES + pl.i;
+        __syncthreads();
     };
-    if (bt.order == 3) {
-        grid_stride_rhs_warps(g.Vh, bt, site);
-    } else if (bt.order == 2) {  // grid-stride sweep: all blocks move through the lattice together, so
-                                 // every right-hand side's neighbours stay in L2 while the band passes
-        for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < g.Vh; h += gridDim.x * blockDim.x)
-            for (int k = 0; k < bt.nrhs; k++) {
-                if (bt.rdone && bt.rdone[k * bt.rdone_stride]) continue;
-                site(h, k);
-            }
-    } else if (bt.order == 1) {  // each right-hand side over the block's chunk, one after another
-        for (int k = 0; k < bt.nrhs; k++) {
-            if (bt.rdone && bt.rdone[k * bt.rdone_stride]) continue;
-            for (int h = blockIdx.x * chunk + threadIdx.x; h < h_end; h += blockDim.x) site(h, k);
+    // kappa^2 A^-1, per spin sign g A^-1 = [[a - i kp g, kpp], [kpp, a + i kp g]] / det
+    const float a = st.kappa2 * st.inv_det, e = a * st.kpp;
+    const float b0 = a * (DAG ? -st.kp : st.kp) * (f == 0 ? 1.0f : -1.0f);
+    walk<RP>(ntile, bt, tile, [&](int k0) {
+        bool on = h < g.Vh;
+        const int k = pl.rhs(k0, bt, on);
+        f2 p[12], o[12];
+        hop_all<DAG, PF, NT, RP>(t, pl.i, s16_at(in, k * bt.stride), f, p);
+#pragma unroll
+        for (int q = 0; q < 12; q++) {
+            const float b = q < 6 ? b0 : -b0;
+            const float x = __shfl_xor_sync(0xffffffffu, p[q].x, 16), y = __shfl_xor_sync(0xffffffffu, p[q].y, 16);
+            o[q] = make_float2(fmaf(a, p[q].x, fmaf(b, p[q].y, e * x)), fmaf(a, p[q].y, fmaf(-b, p[q].x, e * y)));
         }
-    } else {  // every right-hand side of a site before the next site (links hot in cache)
-        for (int h = blockIdx.x * chunk + threadIdx.x; h < h_end; h += blockDim.x)
-            for (int k = 0; k < bt.nrhs; k++) {
-                if (bt.rdone && bt.rdone[k * bt.rdone_stride]) continue;
-                site(h, k);
-            }
-    }
+        store_site(s16_at(out, k * bt.stride), f, min(h, g.Vh - 1), on, o);
+    });
 }
 
-// Per-right-hand-side block partials: each thread keeps its running sums in its own
-// slots of dynamic shared memory, part[(q * nrhs + k) * blockDim + tid], q = 0, 1.
-template <bool DAG, int EPI, bool PF, int NT, int MB>
-__global__ void __launch_bounds__(NT, MB) k_hop_odd_s16(Geom g, SiteTermF st, const int2 *__restrict__ links,
+// Reduction partials: the FP32 sum over 8 threads (4 sites, both flavours; RP = 2: a right-hand side's 16 of the
+// warp) is added in FP64 to a shared slot per (sum, right-hand side, warp and lane).
+template <bool DAG, int EPI, bool PF, int NT, int MB, int RP>
+__global__ void __launch_bounds__(NT, MB) k_hop_odd_s16(LatGeom g, int apbc, SiteTermF st, const int2 *__restrict__ links,
                                                         S16In psi_all, S16In te_all, S16Out out_all, S16EpiArgs ea,
-                                                        int chunk, S16Batch bt) {
-    __shared__ double red[40];
-    __shared__ float alpha_s[TMND_MAX_BATCH];
-    extern __shared__ double part[];
-    if (ea.done && *ea.done) return;
-    const int Vh = g.Vh;
+                                                        int ntile, S16Batch bt) {
     constexpr bool SUMS = EPI == EPI_STORE_NORMS || EPI == EPI_MMS_R;
-    if (EPI == EPI_MMS_R) {
-        if (threadIdx.x < bt.nrhs) alpha_s[threadIdx.x] = (float)ea.alpha[(size_t)threadIdx.x * ea.alpha_stride];
-    }
+    constexpr int NQ = EPI == EPI_STORE_NORMS ? 2 : 1, LANES = RP == 2 ? 1 : 4, SLOTS = NT / 32 * LANES;
+    __shared__ Tile<NT, RP> t;
+    __shared__ double part[SUMS ? NQ * TMND_MAX_BATCH * SLOTS : 1];
+    if (ea.done && *ea.done) return;
+    const Place<RP> pl;
+    const int lane = threadIdx.x & 31, f = pl.f, Vh = g.Vh;
     if (SUMS)
-        for (int k = 0; k < 2 * bt.nrhs; k++) part[k * blockDim.x + threadIdx.x] = 0.0;
-    __syncthreads();
-    const int h_end = min(Vh, (int)(blockIdx.x + 1) * chunk);
-    auto site = [&](int h, int k) {
-        const S16In te = s16_at(te_all, k * bt.stride), psi = s16_at(psi_all, k * bt.stride);
-        const S16Out out = s16_at(out_all, k * bt.stride);
-        f2 acc[4][3][2];
-        hop_all<1, false, PF>(g, links, te.q, te.nrm, h, acc);
-        if constexpr (EPI == EPI_MMS_R) {  // w = y + sigma aux; r' = r - alpha w (FP32 planes), plane by plane
-            const S16In aux = s16_at(ea.aux, k * bt.stride);
-            const float sg = (float)(ea.per_rhs_sigma ? ea.sigma_k[k] : ea.sigma);
-            const float s1 = odd_mms_r_fused<DAG>(st, acc, GSite{psi.q, psi.nrm, h}, GSite{aux.q, aux.nrm, h}, sg,
-                                                  alpha_s[k], ea.r_in + k * ea.r_stride, ea.r + k * ea.r_stride, Vh,
-                                                  h);
-            part[k * blockDim.x + threadIdx.x] += s1;
-            return;
-        }
-        f2 p[4][3][2];
-        load_site(GSite{psi.q, psi.nrm, h}, p);
-        f2 y[4][3][2];
-        float s1 = 0.0f, s2 = 0.0f;
-        odd_term<DAG, EPI == EPI_STORE_NORMS>(st, acc, p, y, s1, s2);
-        if (EPI == EPI_STORE || EPI == EPI_STORE_NORMS) {
-            store_site(out.q, out.nrm, Vh, h, y);
-            if (EPI == EPI_STORE_NORMS) {
-                part[k * blockDim.x + threadIdx.x] += s1;
-                part[(bt.nrhs + k) * blockDim.x + threadIdx.x] += s2;
-            }
-        } else {  // EPI_SHIFT: y + sigma aux
-            const S16In aux = s16_at(ea.aux, k * bt.stride);
-            add_shift(GSite{aux.q, aux.nrm, h}, (float)ea.sigma, y);
-            store_site(out.q, out.nrm, Vh, h, y);
-        }
+        for (int q = threadIdx.x; q < NQ * TMND_MAX_BATCH * SLOTS; q += NT) part[q] = 0.0;
+    int h = 0;
+    auto tile = [&](int w) {
+        __syncthreads();  // the previous tile is done with
+        load_tile<1, NT, RP>(g, apbc, links, w * Tile<NT, RP>::SITES, t);
+        h = w * Tile<NT, RP>::SITES + pl.i;
+        __syncthreads();
     };
-    if (bt.order == 3) {
-        grid_stride_rhs_warps(Vh, bt, site);
-    } else if (bt.order == 2) {
-        for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < Vh; h += gridDim.x * blockDim.x)
-            for (int k = 0; k < bt.nrhs; k++) {
-                if (bt.rdone && bt.rdone[k * bt.rdone_stride]) continue;
-                site(h, k);
-            }
-    } else if (bt.order == 1) {
-        for (int k = 0; k < bt.nrhs; k++) {
-            if (bt.rdone && bt.rdone[k * bt.rdone_stride]) continue;
-            for (int h = blockIdx.x * chunk + threadIdx.x; h < h_end; h += blockDim.x) site(h, k);
+    const float kp0 = (DAG ? -st.kp : st.kp) * (f == 0 ? 1.0f : -1.0f);
+    auto add = [&](float v, int q, int k, bool mine) {
+        v += __shfl_xor_sync(0xffffffffu, v, 16);
+        if (RP == 1) v += __shfl_xor_sync(0xffffffffu, v, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        if (RP == 2) {
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
         }
-    } else {
-        for (int h = blockIdx.x * chunk + threadIdx.x; h < h_end; h += blockDim.x)
-            for (int k = 0; k < bt.nrhs; k++) {
-                if (bt.rdone && bt.rdone[k * bt.rdone_stride]) continue;
-                site(h, k);
+        const int l = RP == 2 ? lane & 7 : lane;  // RP 2: lane 0 holds the first right-hand side's sum, lane 8 the second's
+        if (mine && f == 0 && l < LANES) part[(q * TMND_MAX_BATCH + k) * SLOTS + (threadIdx.x >> 5) * LANES + l] += (double)v;
+    };
+    walk<RP>(ntile, bt, tile, [&](int k0) {
+        bool mine = true;
+        const int k = pl.rhs(k0, bt, mine);
+        const bool on = mine && h < Vh;
+        const S16In te = s16_at(te_all, k * bt.stride), psi = s16_at(psi_all, k * bt.stride);
+        const int hc = min(h, Vh - 1);
+        f2 v[12];
+        hop_all<false, PF, NT, RP>(t, pl.i, te, f, v);
+        Raw own, oth;
+        load_raw(psi, f, hc, own);
+        load_raw(psi, 1 - f, hc, oth);
+        float s1 = 0.0f, s2 = 0.0f;
+        const float sigma = (float)(EPI == EPI_MMS_R && ea.per_rhs_sigma ? ea.sigma_k[k] : ea.sigma);
+        Raw ax;
+        if (EPI == EPI_SHIFT || EPI == EPI_MMS_R) load_raw(s16_at(ea.aux, k * bt.stride), f, hc, ax);
+        const float alpha = EPI == EPI_MMS_R ? (float)ea.alpha[(size_t)k * ea.alpha_stride] : 0.0f;
+#pragma unroll
+        for (int q = 0; q < 12; q++) {
+            // y = A psi - H t (dag: A(-mu) psi - gamma_5 H t)
+            const float b = q < 6 ? kp0 : -kp0;
+            const f2 p = value(own, q, own.nrm), x = value(oth, q, own.nrm);
+            const f2 hp = DAG && q >= 6 ? make_float2(-v[q].x, -v[q].y) : v[q];
+            f2 y = make_float2(fmaf(-b, p.y, fmaf(-st.kpp, x.x, p.x - hp.x)), fmaf(b, p.x, fmaf(-st.kpp, x.y, p.y - hp.y)));
+            if (EPI == EPI_STORE_NORMS) {
+                s1 = fmaf(y.x, y.x, fmaf(y.y, y.y, s1));
+                s2 = fmaf(p.x, p.x, fmaf(p.y, p.y, s2));
             }
-    }
+            if (EPI == EPI_SHIFT || EPI == EPI_MMS_R) {
+                const int w = word(ax, q);
+                const float sa = sigma * ax.nrm;
+                y = make_float2(fmaf(sa, s16_lo(w), y.x), fmaf(sa, s16_hi(w), y.y));
+            }
+            v[q] = y;
+        }
+        if (EPI == EPI_MMS_R) {
+            // r' = r - alpha w: FP32 planes, touched once per launch (evict first); all loads in flight at once
+            const size_t at = (size_t)f * 12 * Vh + hc;
+            const float2 *rin = ea.r_in + k * ea.r_stride + at;
+            float2 *rout = ea.r + k * ea.r_stride + at;
+            float2 r[12];
+#pragma unroll
+            for (int q = 0; q < 12; q++) r[q] = __ldcs(rin + (size_t)q * Vh);
+#pragma unroll
+            for (int q = 0; q < 12; q++) {
+                const float2 r1 = make_float2(fmaf(-alpha, v[q].x, r[q].x), fmaf(-alpha, v[q].y, r[q].y));
+                if (on) __stcs(rout + (size_t)q * Vh, r1);
+                s1 = fmaf(r1.x, r1.x, fmaf(r1.y, r1.y, s1));
+            }
+        }
+        if (EPI != EPI_MMS_R) store_site(s16_at(out_all, k * bt.stride), f, hc, on, v);
+        if (SUMS) add(on ? s1 : 0.0f, 0, k, mine);
+        if (EPI == EPI_STORE_NORMS) add(on ? s2 : 0.0f, 1, k, mine);
+    });
     if (SUMS) {
-        const int nq = EPI == EPI_STORE_NORMS ? 2 : 1;
-        for (int q = 0; q < nq; q++)
-            for (int k = 0; k < bt.nrhs; k++) {
-                const double t = block_sum(part[(q * bt.nrhs + k) * blockDim.x + threadIdx.x], red);
-                if (threadIdx.x == 0) ea.part_out[(size_t)(nq * k + q) * gridDim.x + blockIdx.x] = t;
-                __syncthreads();
-            }
+        __syncthreads();
+        for (int w = threadIdx.x; w < NQ * bt.nrhs; w += NT) {
+            const int q = w / bt.nrhs, k = w - q * bt.nrhs;
+            double s = 0.0;
+            for (int j = 0; j < SLOTS; j++) s += part[(q * TMND_MAX_BATCH + k) * SLOTS + j];
+            ea.part_out[(size_t)(NQ * k + q) * gridDim.x + blockIdx.x] = s;
+        }
     }
 }
 
-template <bool DAG, int EPI, bool PF, int NT, int MB>
-void odd_smem_attr() {
-    static bool done = false;  // dynamic shared memory above 48 KB needs an opt-in (256 threads, 16 RHS)
-    if (!done) {
-        cudaFuncSetAttribute(k_hop_odd_s16<DAG, EPI, PF, NT, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(double) * 2 * TMND_MAX_BATCH * NT));
-        done = true;
-    }
-}
-
-template <bool PF, int NT, int MB>
+template <bool PF, int NT, int MB, int RP>
 int per_sm_of(int dev) {
     int a = 0, b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_hop_odd_s16<true, EPI_MMS_R, PF, NT, MB>, NT,
-                                                  sizeof(double) * 2 * NT);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_hop_even_s16<true, PF, NT, MB>, NT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_hop_odd_s16<true, EPI_MMS_R, PF, NT, MB, RP>, NT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_hop_even_s16<true, PF, NT, MB, RP>, NT, 0);
     a = a < b ? a : b;
     (void)dev;
     return a > 0 ? a : 1;
 }
 
-template <bool PF, int NT, int MB>
+template <bool PF, int NT, int MB, int RP>
 void launch_odd_shape(const Geom &g, const SiteTermF &st, const int2 *links, S16In psi, S16In te, S16Out out,
                       bool dag, HopEpi epi, const S16EpiArgs &ea, cudaStream_t s, const S16Batch &bt, int nb) {
-    const int chunk = (g.Vh + nb - 1) / nb;
-    const size_t smem = sizeof(double) * 2 * bt.nrhs * NT;
-#define TMND_ODD16(D, E)                                                                              \
-    do {                                                                                              \
-        odd_smem_attr<D, E, PF, NT, MB>();                                                            \
-        k_hop_odd_s16<D, E, PF, NT, MB><<<nb, NT, smem, s>>>(g, st, links, psi, te, out, ea, chunk, bt); \
-    } while (0)
+    constexpr int SITES = Tile<NT, RP>::SITES;
+    const int ntile = (g.Vh + SITES - 1) / SITES;
+#define TMND_ODD16(D, E) \
+    k_hop_odd_s16<D, E, PF, NT, MB, RP><<<nb, NT, 0, s>>>(lat_geom(g), g.apbc, st, links, psi, te, out, ea, ntile, bt)
     if (!dag) {
         switch (epi) {
             case EPI_STORE: TMND_ODD16(false, EPI_STORE); break;
@@ -307,17 +347,18 @@ void launch_odd_shape(const Geom &g, const SiteTermF &st, const int2 *links, S16
 }  // namespace
 
 // the extern entry points of one compiled shape (I, threads T, blocks per SM B, prefetch P)
-#define TMND_S16_DEFINE_SHAPE(I, T, B, P)                                                                        \
-    int s16_per_sm_##I() { return per_sm_of<P, T, B>(0); }                                                      \
+#define TMND_S16_DEFINE_SHAPE(I, T, B, P, R)                                                                     \
+    int s16_per_sm_##I() { return per_sm_of<P, T, B, R>(0); }                                                   \
     void s16_even_##I(const Geom &g, const SiteTermF &st, const int2 *links, S16In in, S16Out out, bool dag,    \
                       const int *done, cudaStream_t s, const S16Batch &bt, int nb) {                             \
-        const int chunk = (g.Vh + nb - 1) / nb;                                                                  \
+        const LatGeom lg = lat_geom(g);                                                                          \
+        const int sites = T / (2 * R), ntile = (g.Vh + sites - 1) / sites;                                       \
         if (dag)                                                                                                 \
-            k_hop_even_s16<true, P, T, B><<<nb, T, 0, s>>>(g, st, links, in, out, done, chunk, bt);              \
+            k_hop_even_s16<true, P, T, B, R><<<nb, T, 0, s>>>(lg, g.apbc, st, links, in, out, done, ntile, bt);  \
         else                                                                                                     \
-            k_hop_even_s16<false, P, T, B><<<nb, T, 0, s>>>(g, st, links, in, out, done, chunk, bt);             \
+            k_hop_even_s16<false, P, T, B, R><<<nb, T, 0, s>>>(lg, g.apbc, st, links, in, out, done, ntile, bt); \
     }                                                                                                            \
     void s16_odd_##I(const Geom &g, const SiteTermF &st, const int2 *links, S16In psi, S16In te, S16Out out,     \
                      bool dag, HopEpi epi, const S16EpiArgs &ea, cudaStream_t s, const S16Batch &bt, int nb) {   \
-        launch_odd_shape<P, T, B>(g, st, links, psi, te, out, dag, epi, ea, s, bt, nb);                         \
+        launch_odd_shape<P, T, B, R>(g, st, links, psi, te, out, dag, epi, ea, s, bt, nb);                      \
     }
