@@ -46,40 +46,67 @@ __device__ __forceinline__ void read_site(const void *src, int Vh, int h, float 
     }
 }
 
-// S16 -> F64 keeps the exact dequantised values (scale applied in FP64)
-__global__ void k_s16_to_f64(int Vh, int nrhs, const char *src, char *dst) {
-    const size_t sb = S16_BYTES_PER_SITE * (size_t)Vh, db = sizeof(double2) * 24 * (size_t)Vh;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < (long)Vh * nrhs; i += (long)gridDim.x * blockDim.x) {
-        const int k = (int)(i / Vh), h = (int)(i % Vh);
-        const S16In s = s16_in(src + k * sb, Vh);
-        double2 *d = (double2 *)(dst + k * db);
-        const double sc = s.nrm[s16_ni(h)];
-        for (int j = 0; j < 6; j++) {
-            const int4 w = s.q[s16_qi(j, h)];
-            const int ws[4] = {w.x, w.y, w.z, w.w};
-            for (int m = 0; m < 4; m++)
-                d[(size_t)(4 * j + m) * Vh + h] = make_double2((double)s16_int_lo(ws[m]) * sc, (double)s16_int_hi(ws[m]) * sc);
+// n sc as a double, exactly, n a 16-bit field and sc a positive normal float (bits scb): the product of the
+// mantissas has at most 40 bits and goes straight under the exponent, with no FP64 instruction (at 2 per clock
+// and SM the 96 of a site took longer than its 484 bytes from HBM: 8 right-hand sides at 24^3x48 482 -> 200 us).
+__device__ __forceinline__ double s16_times_scale(int n, unsigned scb) {
+    const unsigned a = (unsigned)abs(n);
+    const int lz = __clz((int)a) - 16;                                    // a << lz in [2^15, 2^16)
+    const unsigned long long p = (unsigned long long)(a << (lz & 31)) * ((scb & 0x7fffffu) | 0x800000u);  // [2^38, 2^40)
+    const int top = (int)(p >> 39);
+    // the leading bit, at 52 after the shift, adds one to the exponent field below it
+    const unsigned long long bits = (p << (14 - top)) + ((unsigned long long)(37 + top - lz + (int)(scb >> 23) - 150 + 1023) << 52);
+    return a ? __longlong_as_double((long long)(bits | (unsigned long long)((unsigned)n & 0x80000000u) << 32)) : 0.0;
+}
+
+// S16 -> F64 keeps the exact dequantised values; right-hand side blockIdx.y
+__global__ void __launch_bounds__(128) k_s16_to_f64(int Vh, const char *src, char *dst) {
+    const int k = blockIdx.y, h = blockIdx.x * blockDim.x + threadIdx.x;
+    if (h >= Vh) return;
+    const S16In s = s16_in(src + k * (S16_BYTES_PER_SITE * (size_t)Vh), Vh);
+    double2 *d = (double2 *)(dst + k * (sizeof(double2) * 24 * (size_t)Vh)) + h;
+    const float sc = s.nrm[s16_ni(h)];
+    const unsigned scb = __float_as_uint(sc);
+    const bool plain = scb - 0x800000u < 0x7f000000u;  // positive, normal, finite
+    int4 q[6];
+#pragma unroll
+    for (int j = 0; j < 6; j++) q[j] = s.q[s16_qi(j, h)];
+    if (!plain) {  // a branch, so that the FP64 instructions are not issued for nothing
+        for (int c = 0; c < 24; c++) {
+            const int w = ((const int *)&s.q[s16_qi(c / 4, h)])[c % 4];
+            d[(size_t)c * Vh] = make_double2((double)s16_int_lo(w) * (double)sc, (double)s16_int_hi(w) * (double)sc);
         }
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < 6; j++) {
+        const int ws[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
+#pragma unroll
+        for (int m = 0; m < 4; m++)
+            d[(size_t)(4 * j + m) * Vh] = make_double2(s16_times_scale(s16_int_lo(ws[m]), scb),
+                                                       s16_times_scale(s16_int_hi(ws[m]), scb));
     }
 }
 
+// right-hand side blockIdx.y
 template <int SRC>
-__global__ void k_to_s16(int Vh, int nrhs, const char *src, size_t src_rhs_bytes, char *dst) {
-    const size_t db = S16_BYTES_PER_SITE * (size_t)Vh;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < (long)Vh * nrhs; i += (long)gridDim.x * blockDim.x) {
-        const int k = (int)(i / Vh), h = (int)(i % Vh);
-        float v[24][2];
-        read_site<SRC>(src + k * src_rhs_bytes, Vh, h, v);
-        float m = 0.0f;
-        for (int c = 0; c < 24; c++) m = fmaxf(m, fmaxf(fabsf(v[c][0]), fabsf(v[c][1])));
-        const float sc = m > 0.0f ? QMAX / m : 0.0f;
-        S16Out o = s16_out(dst + k * db, Vh);
-        o.nrm[s16_ni(h)] = m / QMAX;
-        for (int j = 0; j < 6; j++) {
-            int w[4];
-            for (int q = 0; q < 4; q++) w[q] = s16_pack_fma(v[4 * j + q][0], v[4 * j + q][1], sc);
-            o.q[s16_qi(j, h)] = make_int4(w[0], w[1], w[2], w[3]);
-        }
+__global__ void __launch_bounds__(128) k_to_s16(int Vh, const char *src, size_t src_rhs_bytes, char *dst) {
+    const int k = blockIdx.y, h = blockIdx.x * blockDim.x + threadIdx.x;
+    if (h >= Vh) return;
+    float v[24][2];
+    read_site<SRC>(src + k * src_rhs_bytes, Vh, h, v);
+    float m = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 24; c++) m = fmaxf(m, fmaxf(fabsf(v[c][0]), fabsf(v[c][1])));
+    const float sc = m > 0.0f ? QMAX / m : 0.0f;
+    const S16Out o = s16_out(dst + k * (S16_BYTES_PER_SITE * (size_t)Vh), Vh);
+    o.nrm[s16_ni(h)] = m / QMAX;
+#pragma unroll
+    for (int j = 0; j < 6; j++) {
+        int w[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) w[q] = s16_pack_fma(v[4 * j + q][0], v[4 * j + q][1], sc);
+        o.q[s16_qi(j, h)] = make_int4(w[0], w[1], w[2], w[3]);
     }
 }
 
@@ -145,20 +172,28 @@ size_t spinor_bytes_prec(int Vh, int prec) {
 
 tmnd_status convert_spinor(int Vh, void *dst, int dst_prec, const void *src, int src_prec, int nrhs,
                            cudaStream_t s) {
-    const long nsite = (long)Vh * nrhs;
-    const long nel = 24L * nsite;
+    const long nel = 24L * Vh * nrhs;
+    constexpr int MAX_Y = 65535;  // right-hand sides per launch (the grid's y)
     if (dst_prec == src_prec) {
         TMND_CUDA_TRY(cudaMemcpyAsync(dst, src, spinor_bytes_prec(Vh, src_prec) * nrhs, cudaMemcpyDeviceToDevice, s));
         return TMND_OK;
     }
     if (dst_prec == TMND_S16) {
         const size_t sb = spinor_bytes_prec(Vh, src_prec);
-        if (src_prec == TMND_F64)
-            k_to_s16<TMND_F64><<<grid_for(nsite), 256, 0, s>>>(Vh, nrhs, (const char *)src, sb, (char *)dst);
-        else
-            k_to_s16<TMND_F32><<<grid_for(nsite), 256, 0, s>>>(Vh, nrhs, (const char *)src, sb, (char *)dst);
+        for (int k = 0; k < nrhs; k += MAX_Y) {
+            const dim3 grid((Vh + 127) / 128, nrhs - k < MAX_Y ? nrhs - k : MAX_Y);
+            const char *from = (const char *)src + k * sb;
+            char *to = (char *)dst + k * spinor_bytes_prec(Vh, TMND_S16);
+            if (src_prec == TMND_F64)
+                k_to_s16<TMND_F64><<<grid, 128, 0, s>>>(Vh, from, sb, to);
+            else
+                k_to_s16<TMND_F32><<<grid, 128, 0, s>>>(Vh, from, sb, to);
+        }
     } else if (src_prec == TMND_S16 && dst_prec == TMND_F64) {
-        k_s16_to_f64<<<grid_for(nsite), 256, 0, s>>>(Vh, nrhs, (const char *)src, (char *)dst);
+        for (int k = 0; k < nrhs; k += MAX_Y)
+            k_s16_to_f64<<<dim3((Vh + 127) / 128, nrhs - k < MAX_Y ? nrhs - k : MAX_Y), 128, 0, s>>>(
+                Vh, (const char *)src + k * spinor_bytes_prec(Vh, TMND_S16),
+                (char *)dst + k * spinor_bytes_prec(Vh, TMND_F64));
     } else if (src_prec == TMND_F64 && dst_prec == TMND_F32) {
         k_f64_to_f32<<<grid_for(nel), 256, 0, s>>>(nel, (const double2 *)src, (float2 *)dst);
     } else if (src_prec == TMND_F32 && dst_prec == TMND_F64) {
