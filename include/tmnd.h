@@ -222,7 +222,7 @@ typedef struct {
     int nsolve;            /* the first nsolve shifts must converge; the base system is
                               sigma[nsolve-1]; shifts after it are guess shifts (Sec. 4.2.2)
                               iterated along, never required to converge.  0 = all. */
-    int check_every;       /* iterations between host convergence checks (0 = 32) */
+    int check_every;       /* iterations between host convergence checks (0 = 8) */
     int profile;           /* 1: time the stencil and update kernels of every iteration with
                               CUDA events (filled into hop_ms / update_ms) */
     int prec;              /* TMND_F64 (0): plain FP64 multi-shift CG.

@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_odd_f32(LatGeom g, 
     float2 acc[4][3];
     hop_all<1, false>(g, apbc, links, te + off, h, acc);
     if (hh >= Vh) return;
+    const float sigma = EPI == EPI_SHIFT ? ea.sigma[ea.per_rhs ? blockIdx.y : 0] : 0.0f;
     const float2 *own = psi + off + h, *oth = psi + (size_t)blockIdx.y * NCOMP * Vh + (size_t)(1 - f) * 12 * Vh + h;
     float2 *o = out + off + h;
 #pragma unroll
@@ -184,7 +185,7 @@ __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_odd_f32(LatGeom g, 
             float2 y = make_float2(fmaf(-b, p.y, fmaf(-st.kpp, q.x, p.x - hp.x)), fmaf(b, p.x, fmaf(-st.kpp, q.y, p.y - hp.y)));
             if (EPI == EPI_SHIFT) {
                 const float2 a = __ldg(&ea.aux[off + h + (size_t)(s * 3 + c) * Vh]);
-                y = make_float2(fmaf(ea.sigma, a.x, y.x), fmaf(ea.sigma, a.y, y.y));
+                y = make_float2(fmaf(sigma, a.x, y.x), fmaf(sigma, a.y, y.y));
             }
             o[(s * 3 + c) * Vh] = y;
         }

@@ -341,12 +341,25 @@ tmnd_status apply_f32(tmnd_gauge *g, float2 *out, const float2 *in, int op, doub
         }
         launch_hop_odd_f32(g->geom, g->st, g->links_f32, ik, te, yo, false, EPI_STORE, ea, r, s);
         launch_hop_even_f32(g->geom, g->st, g->links_f32, yo, te, true, r, s);
-        ea.sigma = (float)sigma;
+        ea.sigma[0] = (float)sigma;
         ea.aux = ik;
         launch_hop_odd_f32(g->geom, g->st, g->links_f32, yo, te, ok, true, EPI_SHIFT, ea, r, s);
     }
     TMND_CUDA_TRY(cudaGetLastError());
     return TMND_OK;
+}
+
+// out_k = (Qhat^2 + sigma[k]) in_k for nrhs <= TMND_MAX_BATCH FP32 vectors, all in each launch; te, yo: nrhs each
+void apply_f32_qhat2(tmnd_gauge *g, float2 *out, const float2 *in, const double *sigma, int nrhs, float2 *te, float2 *yo,
+                     cudaStream_t s) {
+    HopEpiArgsF ea = {};
+    launch_hop_even_f32(g->geom, g->st, g->links_f32, in, te, false, nrhs, s);
+    launch_hop_odd_f32(g->geom, g->st, g->links_f32, in, te, yo, false, EPI_STORE, ea, nrhs, s);
+    launch_hop_even_f32(g->geom, g->st, g->links_f32, yo, te, true, nrhs, s);
+    for (int k = 0; k < nrhs; k++) ea.sigma[k] = (float)sigma[k];
+    ea.per_rhs = 1;
+    ea.aux = in;
+    launch_hop_odd_f32(g->geom, g->st, g->links_f32, yo, te, out, true, EPI_SHIFT, ea, nrhs, s);
 }
 
 extern "C" tmnd_status tm_nd_apply(tmnd_gauge *g, void *out, const void *in, int op, double sigma, int nrhs,

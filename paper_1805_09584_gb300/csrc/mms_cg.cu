@@ -63,6 +63,11 @@ struct MMSState {
 };
 
 constexpr int WIN = 8;  // iterations per windowed shift update
+// Iterations per graph replay when the caller leaves it open.  Two replays are queued ahead of the host's read
+// of the done flag, so a solve runs up to three replays' worth of launches past its end (at 32, a third of the
+// launches of the refinement solves, which take 30-60 iterations each); 8 iterations take long enough (0.3 ms
+// on a 4^4 lattice) for the host to keep up, and a quarter of the time to capture.
+constexpr int DEFAULT_CHECK = WIN;
 
 struct MMSCoef {
     int skip;           // the solve was already done before this iteration
@@ -961,8 +966,7 @@ static tmnd_status mms_sloppy(tmnd_gauge *g, const MixedWork &m, const double *s
     tmnd_status ls = run_graph_loop(s, done_all, maxiter, check_every, profile, body, lo);
     if (ls != TMND_OK) return ls;
     hs.resize(R);
-    for (int k = 0; k < R; k++)
-        TMND_CUDA_TRY(cudaMemcpy(&hs[k], (char *)st + k * st_stride, sizeof(MMSState), cudaMemcpyDeviceToHost));
+    TMND_CUDA_TRY(cudaMemcpy2D(hs.data(), sizeof(MMSState), st, st_stride, sizeof(MMSState), R, cudaMemcpyDeviceToHost));
     for (int k = 0; k < R; k++)
         if (hs[k].status == TMND_ERR_NAN) {
             tmnd_set_error("mms_cg_solve: NaN/Inf in a sloppy reduction at iteration %d (right-hand side %d)",
@@ -976,10 +980,11 @@ static tmnd_status mms_sloppy(tmnd_gauge *g, const MixedWork &m, const double *s
 static size_t sloppy_partial_bytes(const Geom &geom, int nrhs) {
     const long n = 24L * geom.Vh;
     const int nb_hop = hop_blocks_s16_max(geom);
-    const int nb_str = stream_blocks(n), nb_site = site_blocks(geom.Vh);
+    const int nb_str = stream_blocks(n), nb_site = site_blocks(geom.Vh), nb_fx = fx_blocks(geom);
     const size_t st_stride = (sizeof(MMSState) + 255) & ~(size_t)255;
     const size_t cf_stride = (sizeof(MMSCoef) + 255) & ~(size_t)255;
-    return sizeof(double) * (size_t)nrhs * (3 * (size_t)nb_hop + (nb_str > nb_site ? nb_str : nb_site)) + 256 +
+    const int nb_one = nb_str > nb_site ? nb_str : nb_site;
+    return sizeof(double) * (size_t)nrhs * (3 * (size_t)nb_hop + (nb_one > nb_fx ? nb_one : nb_fx)) + 256 +
            (size_t)nrhs * (st_stride + cf_stride) + 256;
 }
 
@@ -1032,14 +1037,19 @@ struct DCItem {
 // operator, r = d - (Qhat^2 + sigma) e (accurate to ~1e-7 of |d|, where the 16-bit
 // operator's own ~4e-5 would stall), and r is the next right-hand side.  A pair stops
 // once |r| <= target; the others go on, at most `max_inner` sloppy solves.
-tmnd_status apply_f32(tmnd_gauge *g, float2 *out, const float2 *in, int op, double sigma, int nrhs, int batch,
-                      float2 *te, float2 *yo, cudaStream_t s);
+void apply_f32_qhat2(tmnd_gauge *g, float2 *out, const float2 *in, const double *sigma, int nrhs, float2 *te, float2 *yo,
+                     cudaStream_t s);
 
 // r = d - y (FP32) and block partials |r|^2 (FP64)
+// of right-hand side blockIdx.y (vectors n apart)
 __global__ void k_resid32(long n, const float2 *__restrict__ d, const float2 *__restrict__ y, float2 *__restrict__ r,
                           double *__restrict__ part) {
     __shared__ double red[40];
     double acc = 0.0;
+    d += blockIdx.y * n;
+    y += blockIdx.y * n;
+    r += blockIdx.y * n;
+    part += (size_t)blockIdx.y * gridDim.x;
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
         const float2 u = d[i], v = y[i];
         const float2 w = make_float2(u.x - v.x, u.y - v.y);
@@ -1061,15 +1071,15 @@ __global__ void k_add32(long n, const float2 *__restrict__ c, float2 *__restrict
     }
 }
 
-// FP32 vectors of the inner refinement after the sloppy workspace: d and e per slot, two temporaries
+// FP32 vectors of the inner refinement after the sloppy workspace: d and e per slot
 struct InnerVecs {
-    float2 *d0, *e0, *te, *yo;
+    float2 *d0, *e0;
     long n;
     float2 *d(int c) const { return d0 + (size_t)c * n; }
     float2 *e(int c) const { return e0 + (size_t)c * n; }
 };
 static size_t dc_work_bytes(int Vh, int R) {
-    return mixed_work_bytes(Vh, 1, R) + (2 * (size_t)R + 2) * spinor_bytes_prec(Vh, TMND_F32);
+    return mixed_work_bytes(Vh, 1, R) + 2 * (size_t)R * spinor_bytes_prec(Vh, TMND_F32);
 }
 static InnerVecs inner_vecs(void *base, int Vh, int R) {
     const size_t s32 = spinor_bytes_prec(Vh, TMND_F32);
@@ -1078,8 +1088,6 @@ static InnerVecs inner_vecs(void *base, int Vh, int R) {
     v.n = 24L * Vh;
     v.d0 = (float2 *)w;
     v.e0 = (float2 *)(w + (size_t)R * s32);
-    v.te = (float2 *)(w + 2 * (size_t)R * s32);
-    v.yo = (float2 *)(w + (2 * (size_t)R + 1) * s32);
     return v;
 }
 
@@ -1092,11 +1100,9 @@ static tmnd_status inner_refine(tmnd_gauge *g, const MixedWork &mc, const InnerV
     double *part = (double *)g->partials;
     std::vector<double> rn(dnorm, dnorm + R), tl(R);
     std::vector<int> active(R, 1);
-    std::vector<double> hpart(nb);
-    for (int c = 0; c < R; c++) {
-        TMND_CUDA_TRY(cudaMemcpyAsync(iv.d(c), mc.b32(c), sizeof(float2) * n, cudaMemcpyDeviceToDevice, s));
-        TMND_CUDA_TRY(cudaMemsetAsync(iv.e(c), 0, sizeof(float2) * n, s));
-    }
+    std::vector<double> hpart((size_t)nb * R);
+    TMND_CUDA_TRY(cudaMemcpyAsync(iv.d(0), mc.b32(0), sizeof(float2) * n * R, cudaMemcpyDeviceToDevice, s));
+    TMND_CUDA_TRY(cudaMemsetAsync(iv.e(0), 0, sizeof(float2) * n * R, s));
     for (int j = 0; j < max_inner; j++) {
         int nact = 0;
         for (int c = 0; c < R; c++) {
@@ -1125,21 +1131,22 @@ static tmnd_status inner_refine(tmnd_gauge *g, const MixedWork &mc, const InnerV
             rs.upd_ms += lc.upd_t[k];
         }
         rs.launches += 3 + lc.nlaunch * ((long long)check_every * 7 + check_every / WIN);
-        // accumulate, then the FP32 residual of the accumulated correction as the next right-hand side
+        // accumulate, then the FP32 residuals of the accumulated corrections as the next right-hand sides, all
+        // pairs in each launch and one read of all norms (a pair that has stopped adds zeros and its residual
+        // is not looked at); the ring's and the solution's slots are free until the next solve
+        float2 *te = mc.v.ring0, *yo = mc.v.ring0 + (size_t)R * n;
+        k_add32<<<stream_blocks((long)R * n), UPD_THREADS, 0, s>>>((long)R * n, mc.x32(0, 0), iv.e(0));
+        apply_f32_qhat2(g, yo, iv.e(0), sig, R, te, mc.x32(0, 0), s);
+        k_resid32<<<dim3(nb, R), UPD_THREADS, 0, s>>>(n, iv.d(0), yo, mc.b32(0), part);
+        TMND_CUDA_TRY(cudaMemcpyAsync(hpart.data(), part, sizeof(double) * nb * R, cudaMemcpyDeviceToHost, s));
+        TMND_CUDA_TRY(cudaStreamSynchronize(s));
+        rs.launches += 6;
         for (int c = 0; c < R; c++) {
             if (!active[c]) continue;
-            k_add32<<<nb, UPD_THREADS, 0, s>>>(n, mc.x32(c, 0), iv.e(c));
-            st = apply_f32(g, iv.yo + 0, iv.e(c), TMND_OP_QHAT2, sig[c], 1, 1, iv.te, mc.x32(c, 0), s);
-            if (st != TMND_OK) return st;
-            // apply_f32 left (Qhat^2 + sigma) e in iv.yo (its odd temporary is the slot's x32, free now)
-            k_resid32<<<nb, UPD_THREADS, 0, s>>>(n, iv.d(c), iv.yo, mc.b32(c), part);
-            TMND_CUDA_TRY(cudaMemcpyAsync(hpart.data(), part, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
-            TMND_CUDA_TRY(cudaStreamSynchronize(s));
             double acc = 0;
-            for (int q = 0; q < nb; q++) acc += hpart[q];
+            for (int q = 0; q < nb; q++) acc += hpart[(size_t)c * nb + q];
             rn[c] = sqrt(acc);
             rs.f32 += 1;
-            rs.launches += 5;
             if (!isfinite(rn[c])) {
                 tmnd_set_error("solve: NaN/Inf in an FP32 inner residual (shift %g)", sig[c]);
                 return TMND_ERR_NAN;
@@ -1156,6 +1163,8 @@ static tmnd_status defect_correct(tmnd_gauge *g, void *base, std::vector<DCItem>
     const int Vh = g->geom.Vh;
     const long n = 24L * Vh;
     const int max_rounds = 8;
+    const int nb = fx_blocks(g->geom);  // partials of a defect
+    std::vector<double> hpart;
     tmnd_status st;
     if (max_batch < 1) max_batch = 1;
     if (max_batch > TMND_MAX_BATCH) max_batch = TMND_MAX_BATCH;
@@ -1164,21 +1173,31 @@ static tmnd_status defect_correct(tmnd_gauge *g, void *base, std::vector<DCItem>
         std::vector<DCItem> next;
         size_t q = 0;
         while (q < todo.size()) {
-            // defects of up to max_batch pending pairs, each converted into its sloppy slot
+            // defects of up to max_batch pending pairs, each converted into its sloppy slot, and one host read
+            // of all their norms
             const MixedWork mw = mixed_work(base, Vh, 1, max_batch);
             const InnerVecs iv = inner_vecs(base, Vh, max_batch);
             std::vector<DCItem> chunk;
             std::vector<double> sg, target, dn;
-            for (; q < todo.size() && (int)chunk.size() < max_batch; q++) {
-                DCItem &it = todo[q];
-                double rr = 0;
-                TMND_CUDA_TRY(cudaStreamSynchronize(s));
-                const auto t_f = std::chrono::steady_clock::now();
-                st = fp64_defect(g, mw, it.b, it.x, it.sigma, s, &rr);
+            const int nd = (int)(todo.size() - q) < max_batch ? (int)(todo.size() - q) : max_batch;
+            TMND_CUDA_TRY(cudaStreamSynchronize(s));
+            const auto t_f = std::chrono::steady_clock::now();
+            for (int i = 0; i < nd; i++) {
+                const DCItem &it = todo[q + i];
+                launch_fx_defect(g, it.b, it.x, it.sigma, mw.r64, (double *)g->partials + (size_t)i * nb, mw.fa, mw.fb, s);
+                st = convert_spinor(Vh, mw.b32(i), TMND_F32, mw.r64, TMND_F64, 1, s);
                 if (st != TMND_OK) return st;
-                rs.fp64_ms += ms_since(t_f);  // fp64_defect ends with a host read of its partials
-                rs.fp64++;
-                rs.launches += 5;
+            }
+            hpart.resize((size_t)nd * nb);
+            TMND_CUDA_TRY(cudaMemcpyAsync(hpart.data(), g->partials, sizeof(double) * nd * nb, cudaMemcpyDeviceToHost, s));
+            TMND_CUDA_TRY(cudaStreamSynchronize(s));
+            rs.fp64_ms += ms_since(t_f);
+            rs.fp64 += nd;
+            rs.launches += 6 * nd;
+            for (int i = 0; i < nd; i++) {
+                DCItem &it = todo[q + i];
+                double rr = 0;
+                for (int k = 0; k < nb; k++) rr += hpart[(size_t)i * nb + k];
                 *it.res = sqrt(rr / it.bb);
                 if (round == 0 && it.res0) *it.res0 = *it.res;
                 if (!isfinite(*it.res)) {
@@ -1191,13 +1210,15 @@ static tmnd_status defect_correct(tmnd_gauge *g, void *base, std::vector<DCItem>
                                    it.sigma, max_rounds, *it.res);
                     return TMND_ERR_NOCONV;
                 }
-                st = convert_spinor(Vh, mw.b32((int)chunk.size()), TMND_F32, mw.r64, TMND_F64, 1, s);
-                if (st != TMND_OK) return st;
+                const int slot = (int)chunk.size();  // close the gaps of the pairs that are done
+                if (slot != i)
+                    TMND_CUDA_TRY(cudaMemcpyAsync(mw.b32(slot), mw.b32(i), sizeof(float2) * n, cudaMemcpyDeviceToDevice, s));
                 sg.push_back(it.sigma);
                 target.push_back(0.3 * rho * sqrt(it.bb));  // |d - (Qhat^2 + sigma) e| for |b - ... x'| <= rho |b|
                 dn.push_back(sqrt(rr));
                 chunk.push_back(it);
             }
+            q += nd;
             if (chunk.empty()) continue;
             MixedWork mc = mw;  // the slots the defects were converted into
             mc.nrhs = (int)chunk.size();
@@ -1241,17 +1262,17 @@ static tmnd_status mixed_batch(tmnd_gauge *g, const double2 *b, double2 *const *
     tmnd_status st;
     // |b_k|^2 in FP64
     std::vector<double> bb(R, 0.0);
+    const int nb = stream_blocks(n);
     for (int k = 0; k < R; k++) {
-        const int nb = stream_blocks(n);
-        double *part = (double *)g->partials;
-        k_norm2<<<nb, UPD_THREADS, 0, s>>>(n, b + (size_t)(k0 + k) * n, part);
-        std::vector<double> h(nb);
-        TMND_CUDA_TRY(cudaMemcpyAsync(h.data(), part, sizeof(double) * nb, cudaMemcpyDeviceToHost, s));
-        TMND_CUDA_TRY(cudaStreamSynchronize(s));
-        for (int q = 0; q < nb; q++) bb[k] += h[q];
+        k_norm2<<<nb, UPD_THREADS, 0, s>>>(n, b + (size_t)(k0 + k) * n, (double *)g->partials + (size_t)k * nb);
         st = convert_spinor(Vh, m.b32(k), TMND_F32, b + (size_t)(k0 + k) * n, TMND_F64, 1, s);
         if (st != TMND_OK) return st;
     }
+    std::vector<double> h((size_t)R * nb);
+    TMND_CUDA_TRY(cudaMemcpyAsync(h.data(), g->partials, sizeof(double) * R * nb, cudaMemcpyDeviceToHost, s));
+    TMND_CUDA_TRY(cudaStreamSynchronize(s));
+    for (int k = 0; k < R; k++)
+        for (int q = 0; q < nb; q++) bb[k] += h[(size_t)k * nb + q];
     // 1. batched sloppy multi-shift CG (a zero right-hand side is done at once)
     std::vector<MMSState> hs;
     LoopOut lo;
@@ -1348,7 +1369,7 @@ extern "C" tmnd_status mms_cg_solve(tmnd_gauge *g, const void *b, int nrhs, cons
     TMND_ARG_CHECK(nsolve <= nshift, "mms_cg_solve: nsolve = %d > nshift", nsolve);
     TMND_ARG_CHECK(params->rho > 0 && params->rho < 1, "mms_cg_solve: rho = %g not in (0, 1)", params->rho);
     TMND_ARG_CHECK(params->maxiter >= 1, "mms_cg_solve: maxiter = %d", params->maxiter);
-    int check_every = params->check_every > 0 ? params->check_every : 32;
+    int check_every = params->check_every > 0 ? params->check_every : DEFAULT_CHECK;
     TMND_ARG_CHECK(check_every <= 4096, "mms_cg_solve: check_every too large");
     check_every = (check_every + WIN - 1) / WIN * WIN;  // whole windows per graph replay
 
@@ -1528,6 +1549,8 @@ extern "C" tmnd_status tmnd_hybrid_solve(tmnd_gauge *g, tmnd_mg *mg, const void 
     const int dc_batch = nrhs < TMND_MAX_BATCH ? nrhs : TMND_MAX_BATCH;
     st = tmnd_ensure_workspace(g, dc_work_bytes(Vh, dc_batch));
     if (st != TMND_OK) return st;
+    st = tmnd_ensure_partials(g, sloppy_partial_bytes(g->geom, dc_batch));
+    if (st != TMND_OK) return st;
     const long nfull = 2 * n;  // full-lattice FP32 doublet (complex numbers)
     const size_t f32b = sizeof(float2) * nfull;
     const size_t fxb = fx_bytes(Vh);
@@ -1665,7 +1688,7 @@ extern "C" tmnd_status tmnd_hybrid_solve(tmnd_gauge *g, tmnd_mg *mg, const void 
         if (res_status != TMND_OK) break;
         // FP64 defect correction of this shift's pairs to rho, all right-hand sides together
         RefineStats rs;
-        st = defect_correct(g, g->work, items, hp->rho, rho_inner, hp->maxiter, 32, 0, s, rs, dc_batch);
+        st = defect_correct(g, g->work, items, hp->rho, rho_inner, hp->maxiter, DEFAULT_CHECK, 0, s, rs, dc_batch);
         if (st != TMND_OK) { res_status = st; break; }
         if (hinfo) {
             if (!mg) hinfo->guess_res[i] = res0[0];  // the guess's residual: the first FP64 defect

@@ -143,9 +143,11 @@ enum HopEpi {
     EPI_MMS_R = 3         // w = y + sigma * aux; r -= alpha w; partial |r|^2
 };
 
+constexpr int TMND_MAX_BATCH = 16;
 struct HopEpiArgsF {
-    float sigma;
-    const float2 *aux;      // EPI_SHIFT: the vector multiplied by sigma
+    float sigma[TMND_MAX_BATCH];  // EPI_SHIFT: sigma[0], or (per_rhs) sigma[k] for right-hand side k
+    int per_rhs;
+    const float2 *aux;            // EPI_SHIFT: the vector multiplied by sigma
 };
 
 // The stencil in FP32 on FP32 planes with 18-real FP32 links (the FP32 operator:
@@ -193,7 +195,6 @@ __host__ __device__ inline S16Out s16_out(void *base, int Vh) {
     return S16Out{(int4 *)base, (float *)base};
 }
 
-constexpr int TMND_MAX_BATCH = 16;
 struct S16EpiArgs {
     double sigma;
     // EPI_MMS_R with per_rhs_sigma: right-hand side k uses sigma_k[k] instead of sigma
