@@ -14,6 +14,7 @@
 // are live: 128 registers and 16 warps per SM, where one thread for both flavours took 255 (Qhat^2 at
 // 24^3x48: 488 -> 319 us against 216 us of HBM time; 5 and 6 blocks per SM spill: 435, 447 us).
 #include "lattice.cuh"
+#include "launch.cuh"
 
 namespace {
 
@@ -137,6 +138,7 @@ __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_even_f32(LatGeom g,
                                                                      const float2 *__restrict__ links,
                                                                      const float2 *__restrict__ psi,
                                                                      float2 *__restrict__ out) {
+    dependent_begin();
     const int lane = threadIdx.x & 31, f = lane >> 4, Vh = g.Vh;
     const int hh = (blockIdx.x * (F32_THREADS / 32) + (threadIdx.x >> 5)) * 16 + (lane & 15), h = min(hh, Vh - 1);
     const size_t off = (size_t)blockIdx.y * NCOMP * Vh + (size_t)f * 12 * Vh;
@@ -163,6 +165,7 @@ __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_odd_f32(LatGeom g, 
                                                                     const float2 *__restrict__ psi,
                                                                     const float2 *__restrict__ te,
                                                                     float2 *__restrict__ out, HopEpiArgsF ea) {
+    dependent_begin();
     const int lane = threadIdx.x & 31, f = lane >> 4, Vh = g.Vh;
     const int hh = (blockIdx.x * (F32_THREADS / 32) + (threadIdx.x >> 5)) * 16 + (lane & 15), h = min(hh, Vh - 1);
     const size_t off = (size_t)blockIdx.y * NCOMP * Vh + (size_t)f * 12 * Vh;
@@ -227,6 +230,7 @@ template <int NF>
 __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_dnd(LatGeom g, int apbc, float kappa, float kp, float kpp,
                                                                 float so, const float2 *__restrict__ links,
                                                                 const float2 *__restrict__ in, float2 *__restrict__ out) {
+    dependent_begin();
     if (blockIdx.y == 0) dnd_sites<NF, 0>(g, apbc, kappa, kp, kpp, so, links, in, out);
     else dnd_sites<NF, 1>(g, apbc, kappa, kp, kpp, so, links, in, out);
 }
@@ -240,9 +244,9 @@ void launch_hop_even_f32(const Geom &g, const SiteTerm &st, const float2 *links,
     const dim3 grid(blocks_of(g.Vh, F32_THREADS / 2), nrhs);
     const SiteTerm32 t = site32(st, dag);
     if (dag)
-        k_even_f32<true><<<grid, F32_THREADS, 0, s>>>(lat_geom(g), g.apbc, t, links, psi_o, t_e);
+        launch_dependent(k_even_f32<true>, grid, F32_THREADS, s, lat_geom(g), g.apbc, t, links, psi_o, t_e);
     else
-        k_even_f32<false><<<grid, F32_THREADS, 0, s>>>(lat_geom(g), g.apbc, t, links, psi_o, t_e);
+        launch_dependent(k_even_f32<false>, grid, F32_THREADS, s, lat_geom(g), g.apbc, t, links, psi_o, t_e);
 }
 
 void launch_hop_odd_f32(const Geom &g, const SiteTerm &st, const float2 *links, const float2 *psi_o,
@@ -250,7 +254,7 @@ void launch_hop_odd_f32(const Geom &g, const SiteTerm &st, const float2 *links, 
                         cudaStream_t s) {
     const dim3 grid(blocks_of(g.Vh, F32_THREADS / 2), nrhs);
     const SiteTerm32 t = site32(st, dag);
-#define TMND_ODD32(D, E) k_odd_f32<D, E><<<grid, F32_THREADS, 0, s>>>(lat_geom(g), g.apbc, t, links, psi_o, t_e, y_o, ea)
+#define TMND_ODD32(D, E) launch_dependent(k_odd_f32<D, E>, grid, F32_THREADS, s, lat_geom(g), g.apbc, t, links, psi_o, t_e, y_o, ea)
     if (epi == EPI_STORE) {
         dag ? TMND_ODD32(true, EPI_STORE) : TMND_ODD32(false, EPI_STORE);
     } else {
@@ -262,9 +266,9 @@ void launch_hop_odd_f32(const Geom &g, const SiteTerm &st, const float2 *links, 
 void launch_dnd_full(const Geom &g, double kappa, float kp, float kpp, float s_odd, const float2 *links,
                      const float2 *in, float2 *out, int nf, cudaStream_t s) {
     if (nf == 2)
-        k_dnd<2><<<dim3(blocks_of(g.Vh, F32_THREADS / 2), 2), F32_THREADS, 0, s>>>(lat_geom(g), g.apbc, (float)kappa, kp,
+        launch_dependent(k_dnd<2>, dim3(blocks_of(g.Vh, F32_THREADS / 2), 2), F32_THREADS, s, lat_geom(g), g.apbc, (float)kappa, kp,
                                                                                   kpp, s_odd, links, in, out);
     else
-        k_dnd<1><<<dim3(blocks_of(g.Vh, F32_THREADS), 2), F32_THREADS, 0, s>>>(lat_geom(g), g.apbc, (float)kappa, kp, kpp,
+        launch_dependent(k_dnd<1>, dim3(blocks_of(g.Vh, F32_THREADS), 2), F32_THREADS, s, lat_geom(g), g.apbc, (float)kappa, kp, kpp,
                                                                               s_odd, links, in, out);
 }

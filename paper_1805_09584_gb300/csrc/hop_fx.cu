@@ -24,6 +24,7 @@
 #include <math.h>
 
 #include "hop_fx.cuh"
+#include "launch.cuh"
 #include "lattice.cuh"
 
 namespace {
@@ -281,6 +282,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_even(LatGeom g, Fx
                                                                    FxIn psi, FxOut out, const int *__restrict__ done,
                                                                    int nrun, FxBatch bt) {
     __shared__ FxShared sm;
+    dependent_begin();
     if (done && *done) return;
     psi = fx_next(psi, blockIdx.y * bt.stride);
     out = fx_next(out, blockIdx.y * bt.stride);
@@ -330,6 +332,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_odd(LatGeom g, FxS
                                                                   FxIn psi, FxIn te, FxOdd ea, int nrun, FxBatch bt) {
     __shared__ FxShared sm;
     __shared__ double red[40];
+    dependent_begin();
     if (ea.done && *ea.done) return;
     psi = fx_next(psi, blockIdx.y * bt.stride);
     te = fx_next(te, blockIdx.y * bt.stride);
@@ -472,6 +475,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_odd(LatGeom g, FxS
 
 // FP64 planes -> digits
 __global__ void __launch_bounds__(128) k_fx_from_f64(int Vh, const double2 *__restrict__ in, FxOut out, FxBatch bt) {
+    dependent_begin();
     in += blockIdx.y * bt.n64;
     out = fx_next(out, blockIdx.y * bt.stride);
     const int lane = threadIdx.x & 31, f = lane >> 4;
@@ -505,6 +509,7 @@ __global__ void __launch_bounds__(256) k_fx_to_f32(int Vh, double a, FxIn in, fl
 __global__ void __launch_bounds__(128) k_fx_pupdate(int Vh, const int *__restrict__ skip,
                                                     const double *__restrict__ beta_p,
                                                     const double2 *__restrict__ r, FxOut p) {
+    dependent_begin();
     if (*skip) return;
     const double beta = *beta_p;
     const int lane = threadIdx.x & 31, f = lane >> 4;
@@ -620,7 +625,7 @@ int fx_batch(const Geom &g, int nrhs) {
 
 void launch_fx_from_f64(const Geom &g, const double2 *in, FxOut out, cudaStream_t s, const FxBatch &bt) {
     const int groups = (g.Vh + 15) / 16;
-    k_fx_from_f64<<<dim3((groups + 3) / 4, bt.nrhs), 128, 0, s>>>(g.Vh, in, out, bt);
+    launch_dependent(k_fx_from_f64, dim3((groups + 3) / 4, bt.nrhs), 128, s, g.Vh, in, out, bt);
 }
 
 void launch_fx_to_f32(const Geom &g, double a, FxIn in, float2 *out, cudaStream_t s) {
@@ -630,7 +635,7 @@ void launch_fx_to_f32(const Geom &g, double a, FxIn in, float2 *out, cudaStream_
 void launch_fx_pupdate(const Geom &g, const int *skip, const double *beta, const double2 *r, FxOut p,
                        cudaStream_t s) {
     const int groups = (g.Vh + 15) / 16;
-    k_fx_pupdate<<<(groups + 3) / 4, 128, 0, s>>>(g.Vh, skip, beta, r, p);
+    launch_dependent(k_fx_pupdate, dim3((groups + 3) / 4), 128, s, g.Vh, skip, beta, r, p);
 }
 
 void launch_fx_pack_links(const Geom &g, const double2 *canon, int4 *out, cudaStream_t s) {
@@ -643,9 +648,9 @@ void launch_fx_even(const Geom &g, const FxSite &st, const int4 *links, FxIn psi
     const FxGrid gr = fx_grid(g.Vh);
     const LatGeom fg = lat_geom(g);
     if (dag)
-        k_fx_even<true><<<dim3(gr.blocks, bt.nrhs), FX_THREADS, 0, s>>>(fg, st, links, psi, out, done, gr.runs, bt);
+        launch_dependent(k_fx_even<true>, dim3(gr.blocks, bt.nrhs), FX_THREADS, s, fg, st, links, psi, out, done, gr.runs, bt);
     else
-        k_fx_even<false><<<dim3(gr.blocks, bt.nrhs), FX_THREADS, 0, s>>>(fg, st, links, psi, out, done, gr.runs, bt);
+        launch_dependent(k_fx_even<false>, dim3(gr.blocks, bt.nrhs), FX_THREADS, s, fg, st, links, psi, out, done, gr.runs, bt);
 }
 
 void launch_fx_odd(const Geom &g, const FxSite &st, const int4 *links, FxIn psi, FxIn te, bool dag, FxEpi epi,
@@ -656,7 +661,7 @@ void launch_fx_odd(const Geom &g, const FxSite &st, const int4 *links, FxIn psi,
         ea.sig_e = exponent_of(ea.sigma);
         ea.sig = digits(ea.sigma, ea.sig_e);
     }
-#define TMND_FX(D, E) k_fx_odd<D, E><<<dim3(gr.blocks, bt.nrhs), FX_THREADS, 0, s>>>(fg, st, links, psi, te, ea, gr.runs, bt)
+#define TMND_FX(D, E) launch_dependent(k_fx_odd<D, E>, dim3(gr.blocks, bt.nrhs), FX_THREADS, s, fg, st, links, psi, te, ea, gr.runs, bt)
     switch (epi) {
         case FX_STORE: dag ? TMND_FX(true, FX_STORE) : TMND_FX(false, FX_STORE); break;
         case FX_STORE_NORMS: TMND_FX(false, FX_STORE_NORMS); break;

@@ -37,6 +37,7 @@
 #pragma once
 
 #include "lattice.cuh"
+#include "launch.cuh"
 #include "s16_hop.cuh"
 
 namespace {
@@ -183,6 +184,7 @@ __global__ void __launch_bounds__(NT, MB) k_hop_even_s16(LatGeom g, int apbc, Si
                                                          S16In in, S16Out out, const int *__restrict__ done, int ntile,
                                                          S16Batch bt) {
     __shared__ Tile<NT, RP> t;
+    dependent_begin();
     if (done && *done) return;
     const Place<RP> pl;
     const int f = pl.f;
@@ -221,6 +223,7 @@ __global__ void __launch_bounds__(NT, MB) k_hop_odd_s16(LatGeom g, int apbc, Sit
     constexpr int NQ = EPI == EPI_STORE_NORMS ? 2 : 1, LANES = RP == 2 ? 1 : 4, SLOTS = NT / 32 * LANES;
     __shared__ Tile<NT, RP> t;
     __shared__ double part[SUMS ? NQ * TMND_MAX_BATCH * SLOTS : 1];
+    dependent_begin();
     if (ea.done && *ea.done) return;
     const Place<RP> pl;
     const int lane = threadIdx.x & 31, f = pl.f, Vh = g.Vh;
@@ -325,7 +328,7 @@ void launch_odd_shape(const Geom &g, const SiteTermF &st, const int2 *links, S16
     constexpr int SITES = Tile<NT, RP>::SITES;
     const int ntile = (g.Vh + SITES - 1) / SITES;
 #define TMND_ODD16(D, E) \
-    k_hop_odd_s16<D, E, PF, NT, MB, RP><<<nb, NT, 0, s>>>(lat_geom(g), g.apbc, st, links, psi, te, out, ea, ntile, bt)
+    launch_dependent_if(ntile <= nb, k_hop_odd_s16<D, E, PF, NT, MB, RP>, dim3(nb), NT, s, lat_geom(g), g.apbc, st, links, psi, te, out, ea, ntile, bt)
     if (!dag) {
         switch (epi) {
             case EPI_STORE: TMND_ODD16(false, EPI_STORE); break;
@@ -346,6 +349,8 @@ void launch_odd_shape(const Geom &g, const SiteTermF &st, const int2 *links, S16
 
 }  // namespace
 
+// Launches overlap with the kernel before them only on lattices with at most a tile per block: where the blocks
+// fill the chip for several tiles, the waiting blocks of the next launch cost 2 % (8 right-hand sides, 24^3x48).
 // the extern entry points of one compiled shape (I, threads T, blocks per SM B, prefetch P)
 #define TMND_S16_DEFINE_SHAPE(I, T, B, P, R)                                                                     \
     int s16_per_sm_##I() { return per_sm_of<P, T, B, R>(0); }                                                   \
@@ -354,9 +359,9 @@ void launch_odd_shape(const Geom &g, const SiteTermF &st, const int2 *links, S16
         const LatGeom lg = lat_geom(g);                                                                          \
         const int sites = T / (2 * R), ntile = (g.Vh + sites - 1) / sites;                                       \
         if (dag)                                                                                                 \
-            k_hop_even_s16<true, P, T, B, R><<<nb, T, 0, s>>>(lg, g.apbc, st, links, in, out, done, ntile, bt);  \
+            launch_dependent_if(ntile <= nb, k_hop_even_s16<true, P, T, B, R>, dim3(nb), T, s, lg, g.apbc, st, links, in, out, done, ntile, bt);  \
         else                                                                                                     \
-            k_hop_even_s16<false, P, T, B, R><<<nb, T, 0, s>>>(lg, g.apbc, st, links, in, out, done, ntile, bt); \
+            launch_dependent_if(ntile <= nb, k_hop_even_s16<false, P, T, B, R>, dim3(nb), T, s, lg, g.apbc, st, links, in, out, done, ntile, bt); \
     }                                                                                                            \
     void s16_odd_##I(const Geom &g, const SiteTermF &st, const int2 *links, S16In psi, S16In te, S16Out out,     \
                      bool dag, HopEpi epi, const S16EpiArgs &ea, cudaStream_t s, const S16Batch &bt, int nb) {   \
