@@ -61,6 +61,8 @@ __device__ __forceinline__ void pair_of(int p, int &i0, int &i1, int &s, int &c)
     }
 }
 
+__device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
 __device__ __forceinline__ void copy_async8(void *dst, const void *src, bool valid) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(valid ? 8 : 0));
@@ -141,6 +143,14 @@ __global__ void __launch_bounds__(TR_THREADS, 2) k_restrict(TrGeom g, const floa
         }
         __syncthreads();
         const float2 *cV = sV + (ch & 1) * (NC * TR_ELEMS) + lane;
+        // P's part of the next chunk is on its way while this one is worked on (16 warps per SM alone do not
+        // cover the latency: half the stalls waited for P)
+        const int inext = (ch + 1) * TR_ELEMS + lane;
+#pragma unroll
+        for (int j = 0; j < TR_ELEMS / 32; j++)
+#pragma unroll
+            for (int r = 0; r < RK; r++)
+                if (inext + j * 32 < len) prefetch_l1(&Pr[r][inext + j * 32]);
 #pragma unroll 3
         for (int j = 0; j < TR_ELEMS / 32; j++) {
             const int i = ch * TR_ELEMS + j * 32 + lane;
@@ -198,6 +208,14 @@ __global__ void __launch_bounds__(TR_THREADS) k_prolong(TrGeom g, const float2 *
         float2 acc[2][NC];
 #pragma unroll
         for (int j = 0; j < NC; j++) acc[0][j] = acc[1][j] = make_float2(0.f, 0.f);
+        if (p + TR_THREADS < len / 2) {  // the next pair's elements on their way
+            int n0, n1, ns, nc;
+            pair_of<ZPAIR>(p + TR_THREADS, n0, n1, ns, nc);
+            for (int k = 0; k < g.nv; k++) {
+                prefetch_l1(&Pb[(size_t)k * len + n0]);
+                if (ZPAIR) prefetch_l1(&Pb[(size_t)k * len + n1]);
+            }
+        }
 #pragma unroll 4
         for (int k = 0; k < g.nv; k++) {
             const float2 a0 = __ldg(&Pb[(size_t)k * len + i0]), a1 = __ldg(&Pb[(size_t)k * len + i1]);
