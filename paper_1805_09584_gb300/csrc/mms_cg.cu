@@ -42,7 +42,7 @@
 #include <chrono>
 #include <vector>
 
-#include "hop_fx.cuh"
+#include "fx_sum.cuh"
 #include "launch.cuh"
 
 namespace {
@@ -85,12 +85,10 @@ struct MMSConst {
     double rho2;        // rho^2
 };
 
-template <typename T>
-struct ShiftPtrsT {
-    T *x[NS];
-    T *p[NS];
+struct ShiftPtrs {
+    double2 *x[NS];
+    double2 *p[NS];
 };
-using ShiftPtrs = ShiftPtrsT<double2>;
 
 __global__ void k_init(long n, const double2 *__restrict__ b, double2 *__restrict__ r, ShiftPtrs sp,
                        int nshift, double *__restrict__ part) {
@@ -279,63 +277,110 @@ __global__ void k_alpha(MMSState *st, size_t st_stride, const double *__restrict
 // in the window, x_i += a p_i + sum_l e_l r_l and p_i = P p_i + sum_l Q_l r_l
 // over the WIN residuals of the window.  The dominant HBM stream of the
 // iteration at many shifts, now once per WIN iterations.
-template <typename T>
-struct RingPtrsT {
-    const T *r[WIN];
+struct RingPtrs {
+    const double2 *r[WIN];
 };
-using RingPtrs = RingPtrsT<double2>;
 
-// T = double2 (FP64 path) or float2 (sloppy path; coefficients rounded to FP32)
-template <typename T>
-__global__ void __launch_bounds__(UPD_THREADS) k_window(long n, const MMSCoef *__restrict__ cf, RingPtrsT<T> ring,
-                                                        ShiftPtrsT<T> sp, int nshift) {
-    __shared__ double s_P[NS], s_a[NS], s_Q[NS][WIN], s_e[NS][WIN];
-    __shared__ int s_idx[NS];
+// Bound by the FP64 pipe when the sums run on it (18 multiply-adds per component and shift for 32 bytes).  They run
+// on the integer pipe (fx_sum.cuh): the residuals become words once for all shifts, p_i per shift under its own
+// exponent; what is left to the FP64 pipe is the conversion of the two sums and the addition to x_i.
+// 16^3x32, 12 shifts (mean over a solve's 23 windows): 511 us on the FP64 pipe, 330 us so, 358 us with p_i's terms
+// in FP64.  Against extended precision, a whole solve with 12 shifts of 1e-5..2: every window's x_i has 0.2 to
+// 0.7 times the error of the FP64 chain.
+__global__ void __launch_bounds__(UPD_THREADS, 2) k_window(long n, const MMSCoef *__restrict__ cf, RingPtrs ring,
+                                                           ShiftPtrs sp, int nshift) {
+    __shared__ FxWeight s_w[NS][2][WIN + 1];  // e_l and a, Q_l and P
+    __shared__ int s_e[NS][2], s_ep[NS][2];   // exponents of the sums' units: over l, p_i's term
+    __shared__ int s_idx[NS], s_fx[NS], s_used[WIN];
     __shared__ int s_n;
     dependent_begin();
+    if (threadIdx.x < WIN) s_used[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         int m = 0;
         for (int s = 0; s < nshift; s++)
-            if (cf->touched[s]) {
-                s_idx[m] = s;
-                s_P[m] = cf->P[s];
-                s_a[m] = cf->a[s];
-                for (int l = 0; l < WIN; l++) {
-                    s_Q[m][l] = cf->Q[s][l];
-                    s_e[m][l] = cf->e[s][l];
-                }
-                m++;
-            }
+            if (cf->touched[s]) s_idx[m++] = s;
         s_n = m;
     }
     __syncthreads();
     const int m = s_n;
     if (m == 0) return;
-    using R = decltype(T::x);
+    if (threadIdx.x < m) {
+        const int k = threadIdx.x, s = s_idx[k];
+        bool ok = true;
+        for (int q = 0; q < 2; q++) {
+            const double *w = q ? cf->Q[s] : cf->e[s];
+            const double wp = q ? cf->P[s] : cf->a[s];
+            double mx = 0.0;
+            for (int l = 0; l < WIN; l++) {
+                ok = ok && isfinite(w[l]);
+                mx = fmax(mx, fabs(w[l]));
+                if (w[l] != 0.0) s_used[l] = 1;
+            }
+            int e = 0, ep = 0;
+            frexp(mx, &e);
+            frexp(wp, &ep);
+            ok = ok && isfinite(wp) && abs(e) <= FXW_EXP && abs(ep) <= FXW_EXP && (mx != 0.0 || wp != 0.0);
+            // a sum that is zero throughout does not set the common unit
+            s_e[k][q] = mx != 0.0 ? e - FX_SUM_BITS : -10000;
+            s_ep[k][q] = wp != 0.0 ? ep - FX_SUM_BITS : -10000;
+            if (ok) {
+                for (int l = 0; l < WIN; l++) s_w[k][q][l] = fx_weight(w[l], e);
+                s_w[k][q][WIN] = fx_weight(wp, ep);
+            }
+        }
+        s_fx[k] = ok;
+    }
+    __syncthreads();
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        T rv[WIN];
+        int h[2][WIN], l[2][WIN], er[2];
+        bool fx;
+        {
+            double v[2][WIN];
 #pragma unroll
-        for (int l = 0; l < WIN; l++) rv[l] = ring.r[l][i];
+            for (int j = 0; j < WIN; j++) {  // slots past the solve's end hold no residual of this window
+                const double2 r = s_used[j] ? ring.r[j][i] : make_double2(0.0, 0.0);
+                v[0][j] = r.x;
+                v[1][j] = r.y;
+            }
+            fx = fx_numbers<WIN>(v[0], h[0], l[0], er[0]) && fx_numbers<WIN>(v[1], h[1], l[1], er[1]);
+        }
         for (int k = 0; k < m; k++) {
             const int s = s_idx[k];
-            T *xs = sp.x[s];
-            T *ps = sp.p[s];
-            const T pi = ps[i];
-            T xv = xs[i];
-            T pn;
-            pn.x = (R)s_P[k] * pi.x;
-            pn.y = (R)s_P[k] * pi.y;
-            xv.x = fma((R)s_a[k], pi.x, xv.x);
-            xv.y = fma((R)s_a[k], pi.y, xv.y);
+            double2 *xs = sp.x[s];
+            double2 *ps = sp.p[s];
+            const double2 p0 = ps[i], x0 = xs[i];
+            double p[2] = {p0.x, p0.y}, x[2] = {x0.x, x0.y};
+            int hp[2], lp[2], ep[2];
+            if (fx && s_fx[k] && fx_numbers<1>(&p[0], &hp[0], &lp[0], ep[0]) &&
+                fx_numbers<1>(&p[1], &hp[1], &lp[1], ep[1])) {
 #pragma unroll
-            for (int l = 0; l < WIN; l++) {
-                xv.x = fma((R)s_e[k][l], rv[l].x, xv.x);
-                xv.y = fma((R)s_e[k][l], rv[l].y, xv.y);
-                pn.x = fma((R)s_Q[k][l], rv[l].x, pn.x);
-                pn.y = fma((R)s_Q[k][l], rv[l].y, pn.y);
+                for (int c = 0; c < 2; c++) {
+                    int u;
+                    long long t = fx_add(fx_sum<WIN>(s_w[k][0], h[c], l[c]), s_e[k][0] + er[c],
+                                         fx_sum<1>(&s_w[k][0][WIN], &hp[c], &lp[c]), s_ep[k][0] + ep[c], u);
+                    x[c] = fma((double)t, fx_pow2(u), x[c]);
+                    t = fx_add(fx_sum<WIN>(s_w[k][1], h[c], l[c]), s_e[k][1] + er[c],
+                               fx_sum<1>(&s_w[k][1][WIN], &hp[c], &lp[c]), s_ep[k][1] + ep[c], u);
+                    p[c] = fx_value(t, u);
+                }
+            } else {
+                const double *we = cf->e[s], *wq = cf->Q[s];
+                const double a = cf->a[s], P = cf->P[s];
+                for (int c = 0; c < 2; c++) {
+                    x[c] = fma(a, p[c], x[c]);
+                    p[c] *= P;
+                }
+                for (int j = 0; j < WIN; j++) {
+                    if (!s_used[j]) continue;
+                    const double2 r = ring.r[j][i];
+                    x[0] = fma(we[j], r.x, x[0]);
+                    x[1] = fma(we[j], r.y, x[1]);
+                    p[0] = fma(wq[j], r.x, p[0]);
+                    p[1] = fma(wq[j], r.y, p[1]);
+                }
             }
-            xs[i] = xv;
-            ps[i] = pn;
+            xs[i] = make_double2(x[0], x[1]);
+            ps[i] = make_double2(p[0], p[1]);
         }
     }
 }
@@ -721,7 +766,7 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
         mark(1);
         launch_dependent(k_scalars, dim3(1), SCAL_THREADS, s, st, cf, nb_hop, part_rr, c, j, hist, hist_cap);
         launch_fx_pupdate(g->geom, &cf->skip, &cf->beta, slot[j], p, s);
-        if (j == WIN - 1) launch_dependent(k_window<double2>, dim3(nb_str), UPD_THREADS, s, n, cf, ring, ptrs, nshift);
+        if (j == WIN - 1) launch_dependent(k_window, dim3(nb_str), UPD_THREADS, s, n, cf, ring, ptrs, nshift);
         mark(2);
     };
     LoopOut lo;
