@@ -281,54 +281,54 @@ struct RingPtrs {
     const double2 *r[WIN];
 };
 
+constexpr int WINDOW_BLOCKS = 2;  // per SM, and the grid: a block prepares the coefficients once
 // Bound by the FP64 pipe when the sums run on it (18 multiply-adds per component and shift for 32 bytes).  They run
 // on the integer pipe (fx_sum.cuh): the residuals become words once for all shifts, p_i per shift under its own
 // exponent; what is left to the FP64 pipe is the conversion of the two sums and the addition to x_i.
-// 16^3x32, 12 shifts (mean over a solve's 23 windows): 511 us on the FP64 pipe, 330 us so, 358 us with p_i's terms
-// in FP64.  Against extended precision, a whole solve with 12 shifts of 1e-5..2: every window's x_i has 0.2 to
+// 16^3x32, 12 shifts (mean over a solve's 23 windows): 511 us on the FP64 pipe, 307 us so (358 us with p_i's
+// terms in FP64; 330 us with 8 blocks per SM, each with its coefficients prepared by a thread per shift).  Against extended precision, a whole solve with 12 shifts of 1e-5..2: every window's x_i has 0.2 to
 // 0.7 times the error of the FP64 chain.
-__global__ void __launch_bounds__(UPD_THREADS, 2) k_window(long n, const MMSCoef *__restrict__ cf, RingPtrs ring,
+__global__ void __launch_bounds__(UPD_THREADS, WINDOW_BLOCKS) k_window(long n, const MMSCoef *__restrict__ cf, RingPtrs ring,
                                                            ShiftPtrs sp, int nshift) {
     __shared__ FxWeight s_w[NS][2][WIN + 1];  // e_l and a, Q_l and P
     __shared__ int s_e[NS][2], s_ep[NS][2];   // exponents of the sums' units: over l, p_i's term
-    __shared__ int s_idx[NS], s_fx[NS], s_used[WIN];
+    __shared__ int s_idx[NS], s_ok[NS][2], s_used[WIN];
     __shared__ int s_n;
     dependent_begin();
     if (threadIdx.x < WIN) s_used[threadIdx.x] = 0;
-    if (threadIdx.x == 0) {
-        int m = 0;
-        for (int s = 0; s < nshift; s++)
-            if (cf->touched[s]) s_idx[m++] = s;
-        s_n = m;
+    if (threadIdx.x < 32) {
+        static_assert(NS <= 32, "a lane per shift");
+        const int s = threadIdx.x;
+        const unsigned on = __ballot_sync(0xffffffffu, s < nshift && cf->touched[s]);
+        if (on >> s & 1) s_idx[__popc(on & ((1u << s) - 1))] = s;
+        if (s == 0) s_n = __popc(on);
     }
     __syncthreads();
     const int m = s_n;
     if (m == 0) return;
-    if (threadIdx.x < m) {
-        const int k = threadIdx.x, s = s_idx[k];
-        bool ok = true;
-        for (int q = 0; q < 2; q++) {
-            const double *w = q ? cf->Q[s] : cf->e[s];
-            const double wp = q ? cf->P[s] : cf->a[s];
-            double mx = 0.0;
-            for (int l = 0; l < WIN; l++) {
-                ok = ok && isfinite(w[l]);
-                mx = fmax(mx, fabs(w[l]));
-                if (w[l] != 0.0) s_used[l] = 1;
-            }
-            int e = 0, ep = 0;
-            frexp(mx, &e);
-            frexp(wp, &ep);
-            ok = ok && isfinite(wp) && abs(e) <= FXW_EXP && abs(ep) <= FXW_EXP && (mx != 0.0 || wp != 0.0);
-            // a sum that is zero throughout does not set the common unit
-            s_e[k][q] = mx != 0.0 ? e - FX_SUM_BITS : -10000;
-            s_ep[k][q] = wp != 0.0 ? ep - FX_SUM_BITS : -10000;
-            if (ok) {
-                for (int l = 0; l < WIN; l++) s_w[k][q][l] = fx_weight(w[l], e);
-                s_w[k][q][WIN] = fx_weight(wp, ep);
-            }
+    if (threadIdx.x < 2 * m) {
+        const int k = threadIdx.x >> 1, q = threadIdx.x & 1, s = s_idx[k];
+        const double *w = q ? cf->Q[s] : cf->e[s];
+        const double wp = q ? cf->P[s] : cf->a[s];
+        double mx = 0.0;
+        bool ok = isfinite(wp);
+        for (int l = 0; l < WIN; l++) {
+            ok = ok && isfinite(w[l]);
+            mx = fmax(mx, fabs(w[l]));
+            if (w[l] != 0.0) s_used[l] = 1;
         }
-        s_fx[k] = ok;
+        int e = 0, ep = 0;
+        frexp(mx, &e);
+        frexp(wp, &ep);
+        ok = ok && abs(e) <= FXW_EXP && abs(ep) <= FXW_EXP && (mx != 0.0 || wp != 0.0);
+        // a sum that is zero throughout does not set the common unit
+        s_e[k][q] = mx != 0.0 ? e - FX_SUM_BITS : -10000;
+        s_ep[k][q] = wp != 0.0 ? ep - FX_SUM_BITS : -10000;
+        if (ok) {
+            for (int l = 0; l < WIN; l++) s_w[k][q][l] = fx_weight(w[l], e);
+            s_w[k][q][WIN] = fx_weight(wp, ep);
+        }
+        s_ok[k][q] = ok;
     }
     __syncthreads();
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(UPD_THREADS, 2) k_window(long n, const MMSCoef
             const double2 p0 = ps[i], x0 = xs[i];
             double p[2] = {p0.x, p0.y}, x[2] = {x0.x, x0.y};
             int hp[2], lp[2], ep[2];
-            if (fx && s_fx[k] && fx_numbers<1>(&p[0], &hp[0], &lp[0], ep[0]) &&
+            if (fx && s_ok[k][0] && s_ok[k][1] && fx_numbers<1>(&p[0], &hp[0], &lp[0], ep[0]) &&
                 fx_numbers<1>(&p[1], &hp[1], &lp[1], ep[1])) {
 #pragma unroll
                 for (int c = 0; c < 2; c++) {
@@ -562,13 +562,13 @@ int site_blocks(int Vh) {
     return (int)(want < cap ? want : cap);
 }
 
-int stream_blocks(long n) {
+int stream_blocks(long n, int per_sm = 8) {  // 8 resident 256-thread blocks per SM
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (sms <= 0) sms = 152;
     long want = (n + UPD_THREADS - 1) / UPD_THREADS;
-    long cap = (long)sms * 8;   // 8 resident 256-thread blocks per SM
+    long cap = (long)sms * per_sm;
     return (int)(want < cap ? want : cap);
 }
 
@@ -721,6 +721,7 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
     }
     // small device area after the partials
     const int nb_hop = fx_blocks(g->geom);
+    const int nb_win = stream_blocks(n, WINDOW_BLOCKS);
     const int nb_str = stream_blocks(n);
     double *part_norm = (double *)g->partials;              // 2 * nb_hop
     double *part_rr = part_norm + 2 * nb_hop;               // nb_hop
@@ -766,7 +767,7 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
         mark(1);
         launch_dependent(k_scalars, dim3(1), SCAL_THREADS, s, st, cf, nb_hop, part_rr, c, j, hist, hist_cap);
         launch_fx_pupdate(g->geom, &cf->skip, &cf->beta, slot[j], p, s);
-        if (j == WIN - 1) launch_dependent(k_window, dim3(nb_str), UPD_THREADS, s, n, cf, ring, ptrs, nshift);
+        if (j == WIN - 1) launch_dependent(k_window, dim3(nb_win), UPD_THREADS, s, n, cf, ring, ptrs, nshift);
         mark(2);
     };
     LoopOut lo;
