@@ -45,7 +45,7 @@ namespace {
 // Launch shapes the kernels are compiled in: threads per block, resident blocks per SM the register budget is
 // cut for, next-direction prefetch, right-hand sides per pass.  The autotuner times each on the GPU per
 // (lattice, right-hand sides per launch) and keeps the fastest; shape 0 is the default.
-#define TMND_S16_SHAPE_LIST(X) X(0, 128, 4, true, 1) X(1, 128, 5, true, 2) X(2, 64, 8, true, 2) X(3, 64, 10, true, 2)
+#define TMND_S16_SHAPE_LIST(X) X(0, 128, 4, true, 1) X(1, 128, 5, true, 2) X(2, 64, 8, true, 2) X(3, 64, 7, true, 2)
 
 template <int NT, int RP>
 struct Tile {
