@@ -86,13 +86,13 @@ GAUGE_SEED, RHS_SEED = 1002, 2032
 
 # Algorithmic counts per odd site for ONE FP64 stencil launch (both flavours):
 #   flops: 2 x 1320 (Wilson hop with spin projection, 8 directions) + 240 (A^-1 or A site term)
-#   bytes (FP64, 18-real links): even launch 240 reals (in 48, links 144, out 48),
+#   bytes (8 per real, 18-real links): even launch 240 reals (in 48, links 144, out 48),
 #   odd launch 288 reals (t 48, psi 48, links 144, out 48)
 HOP_FLOP_PER_SITE = 2 * 1320 + 240
 HOP_BYTES_PER_SITE = (240 + 288) / 2 * 8
-# DRAM bytes of one odd-site FP64 stencil launch at 16^3x32, one ncu capture of this kernel
-# (dram__bytes_read.sum + dram__bytes_write.sum: 132.87 MB + 9.04 MB)
-FP64_ODD_LAUNCH_TRAFFIC = 132.866816e6 + 9.036288e6
+# DRAM bytes of one odd-site FP64 stencil launch (k_fx_odd) at 16^3x32, one ncu capture of this kernel
+# (dram__bytes_read.sum + dram__bytes_write.sum)
+FP64_ODD_LAUNCH_TRAFFIC = 129.56e6 + 10.95e6
 FP64_TRAFFIC_VH = 65536
 # 16-bit stencil, algorithmic bytes per odd site and right-hand side: even launch 200 (in 100,
 # out 100) + 192 links, odd launch 300 (+ psi 100) + 192 links; a Qhat^2 + sigma is 2 even +
@@ -105,7 +105,7 @@ F32_Q2_BYTES_PER_SITE = 2 * ((192 + 576 + 192) + (192 + 192 + 576 + 192)) + 192
 S16_LINK_BYTES_PER_SITE = 4 * 192
 # DRAM bytes (read + write) of one 16-bit Qhat^2 + sigma, one ncu capture of its 4 launches:
 # {(lattice V/2, RHS per launch): bytes}
-# (the 8-RHS entry: the grid-stride variant the autotuner keeps there, 64 threads x 6 blocks per SM)
+# (of the kernel's earlier form, both flavours per thread; the 8-RHS entry in grid-stride order)
 S16_Q2_TRAFFIC = {(331776, 1): (97.503232e6 + 3.967232e6) + (132.547840e6 + 8.404480e6)
                   + (97.519360e6 + 3.632896e6) + (169.893632e6 + 15.372288e6),
                   (1048576, 8): (3218.8e6 + 820.7e6) + (4144.8e6 + 821.5e6)
@@ -305,23 +305,27 @@ def s16_roofline(tm, g, flush, stream, nrhs=1, reps=20):
 
 def fp64_roofline(tm, g, flush, stream, peak_tflops, reps=10):
     """The FP64 stencil of the true residuals and defect corrections: median CUDA-event
-    time of one FP64 Qhat^2 + sigma (4 launches, 1 RHS) on the form's lattice, against
-    the FP64 throughput measured in this run (FP64-pipe bound on GB300)."""
+    time of one FP64 Qhat^2 + sigma (conversion to fixed point + 4 launches, 1 RHS) on the form's
+    lattice, against the measured copy bandwidth.  The products run on the integer pipe; their
+    rate as FP64 operations is given beside the FP64 throughput measured in this run."""
     import torch
     x = g.pack(torch.randn(g.vh * 24, dtype=torch.complex128, device="cuda").view(1, g.vh, 2, 4, 3))
     y = g.spinor()
     ms = _median_ms(lambda: tm.tm_nd_apply(g.handle, y, x, tm.OP_QHAT2, 0.01, stream=stream), flush, stream, reps)
     tf = 4 * HOP_FLOP_PER_SITE * g.vh / (ms / 1e3) / 1e12
     del x, y
-    return {"bound": "alu", "kernel": "k_hop_even/k_hop_odd (FP64 stencil, Qhat^2 + sigma: 4 launches)",
-            "achieved": tf, "peak": peak_tflops, "unit": "TFLOP/s", "frac": tf / peak_tflops,
+    gbs = 4 * HOP_BYTES_PER_SITE * g.vh / (ms / 1e3) / 1e9
+    peak, src = hbm_peak()
+    return {"bound": "hbm", "kernel": "k_fx_even/k_fx_odd (FP64 stencil in fixed point, Qhat^2 + sigma: 4 launches)",
+            "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak, "peak_source": src,
+            "tflops": tf, "dgemm_tflops": peak_tflops,
+            "dgemm_source": "cuBLAS DGEMM 8192^3 (torch, best of 5) measured in this run",
             "traffic": FP64_ODD_LAUNCH_TRAFFIC * g.vh / FP64_TRAFFIC_VH,
             "traffic_note": "DRAM bytes of one odd-site launch from an ncu capture at 16^3x32, scaled by the "
                             "number of sites",
-            "peak_source": "cuBLAS DGEMM 8192^3 (torch, best of 5) measured in this run",
             "algorithmic_flop_per_launch": HOP_FLOP_PER_SITE * g.vh,
             "measured": f"median of {reps} CUDA-event timings of tm_nd_apply(Qhat^2 + sigma, FP64), L2 flushed",
-            "ms_per_qhat2": ms, "gbs": 4 * HOP_BYTES_PER_SITE * g.vh / (ms / 1e3) / 1e9}
+            "ms_per_qhat2": ms}
 
 
 FORMS = {
@@ -644,8 +648,8 @@ def run_kernel(args):
         y = g.spinor()
         ms = timed(lambda: tm.tm_nd_apply(g.handle, y, x, tm.OP_QHAT2, 0.01, stream=stream))
         tf = 4 * HOP_FLOP_PER_SITE * g.vh / (ms / 1e3) / 1e12
-        out.update(lattice="16^3x32", ms_qhat2=ms, tflops=tf, fp64_peak_tflops=FP64_PEAK_TFLOPS,
-                   frac=tf / FP64_PEAK_TFLOPS, gbs=4 * HOP_BYTES_PER_SITE * g.vh / (ms / 1e3) / 1e9)
+        gbs = 4 * HOP_BYTES_PER_SITE * g.vh / (ms / 1e3) / 1e9
+        out.update(lattice="16^3x32", ms_qhat2=ms, tflops=tf, gbs=gbs, frac=gbs / hbm_peak()[0])
     elif args.kernel == "f32":
         for dims, name in (((48, 24, 24, 24), "24^3x48"), ((64, 32, 32, 32), "32^3x64")):
             g = tm.Gauge(synth.random_su3_field(dims, ROUGHNESS, 1003), dims, KAPPA, MU_BAR, EPS_BAR)
@@ -975,13 +979,6 @@ def run_study_errors(args):
             "normalisation": "|r| and |e| divided by |b|; site norms of e divided by the largest site norm of b",
             "single_systems": "(Qhat + i mu) x_+ = b, exact x_+ = (Qhat - i mu) x", "seconds": time.perf_counter() - t0,
             "rows": rows}
-
-
-
-
-# nominal FP64 rate of a GB300 (sm_103a): 152 SMs x 2 FP64 FMA/clk/SM x 2 flop x 2.07 GHz;
-# the headline's FP64 roofline uses the DGEMM rate measured in the run instead
-FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 
 
 def oracle_full_iters(name):

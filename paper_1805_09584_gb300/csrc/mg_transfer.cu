@@ -9,7 +9,8 @@
 // vectors, 62 us of the FP32 pipes, against 74 us for the 0.5 GB of P and vectors from HBM: P has to be
 // read once for all columns and the products have to come out of registers.  One thread block per (block,
 // chirality); a register tile per thread.  Before, each of the 96 output rows gathered the fine vector
-// again: restriction 2768 us, prolongation 654 us; now 247 and 244 us.
+// again: restriction 2768 us, prolongation 654 us; now 209 and 184 us (247 and 244
+// before P was prefetched into L1).
 //
 // The fine vectors are planes over half-lattice sites: a block's sites are contiguous only along z, two of
 // a parity in a 4-block.  The prolongation therefore writes pairs.  ZPAIR (block extent in z a multiple of

@@ -11,17 +11,18 @@
 //   p_i = zeta_i' r + beta_i p_i;  p = r + beta p
 // and shift i freezes once |zeta_i| |r| <= rho |b| (its residual is zeta_i r).
 //
-// Per iteration the device runs six kernels and never waits for the host:
+// Per iteration the device runs seven kernels and never waits for the host
+// (p, y and t as fixed-point digits, hop_fx.cuh; r, x_i and p_i in FP64):
 //   1 even hop   t = kappa^2 A^-1 H p
 //   2 odd hop    y = Mhat p, with block partials |y|^2, |p|^2
 //                ((p, w) = |Mhat p|^2 + sigma_0 |p|^2, so w is never formed)
-//   3 even hop   t = kappa^2 A(-mu)^-1 H gamma_5 y
-//   4 odd hop    w = Mhat^+ y + sigma_0 p is applied directly: r' = r - alpha w
+//   3 alpha      deterministic sums of the partials, alpha
+//   4 even hop   t = kappa^2 A(-mu)^-1 H gamma_5 y
+//   5 odd hop    w = Mhat^+ y + sigma_0 p is applied directly: r' = r - alpha w
 //                into the next slot of a ring of WIN residuals, block partials |r'|^2
-//   5 scalars    one thread: deterministic sums of the partials, alpha, beta,
-//                zeta_i', alpha_i, beta_i, freezing, done flag, and the window
-//                coefficients below (single state in device memory)
-//   6 p update   p = r' + beta p
+//   6 scalars    a thread per shift: beta, zeta_i', alpha_i, beta_i, freezing, done flag,
+//                and the window coefficients below (single state in device memory)
+//   7 p update   p = r' + beta p
 // Windowed shift update: the shifted vectors are touched once per WIN
 // iterations.  Within a window starting at iteration k0,
 //   p_i^(k0+j) = P_j p_i^(k0) + sum_{l<j} Q_{j,l} r^(k0+l+1)
@@ -286,10 +287,11 @@ constexpr int WINDOW_BLOCKS = 2;  // per SM, and the grid: a block prepares the 
 // on the integer pipe (fx_sum.cuh): the residuals become words once for all shifts, p_i per shift under its own
 // exponent; what is left to the FP64 pipe is the conversion of the two sums and the addition to x_i.
 // 16^3x32, 12 shifts (mean over a solve's 23 windows): 511 us on the FP64 pipe, 307 us so (358 us with p_i's
-// terms in FP64; 330 us with 8 blocks per SM, each with its coefficients prepared by a thread per shift).  Against extended precision, a whole solve with 12 shifts of 1e-5..2: every window's x_i has 0.2 to
-// 0.7 times the error of the FP64 chain.
-__global__ void __launch_bounds__(UPD_THREADS, WINDOW_BLOCKS) k_window(long n, const MMSCoef *__restrict__ cf, RingPtrs ring,
-                                                           ShiftPtrs sp, int nshift) {
+// terms in FP64; 330 us with 8 blocks per SM, each with its coefficients prepared by a thread per shift).
+// Against extended precision, a whole solve with 12 shifts of 1e-5..2: every window's x_i has 0.2 to 0.7 times
+// the error of the FP64 chain.
+__global__ void __launch_bounds__(UPD_THREADS, WINDOW_BLOCKS) k_window(long n, const MMSCoef *__restrict__ cf,
+                                                                       RingPtrs ring, ShiftPtrs sp, int nshift) {
     __shared__ FxWeight s_w[NS][2][WIN + 1];  // e_l and a, Q_l and P
     __shared__ int s_e[NS][2], s_ep[NS][2];   // exponents of the sums' units: over l, p_i's term
     __shared__ int s_idx[NS], s_ok[NS][2], s_used[WIN];
