@@ -470,13 +470,14 @@ __global__ void k_pupdate_s(int Vh, const MMSCoef *__restrict__ cf0, size_t cf_s
 __global__ void __launch_bounds__(UPD_THREADS) k_window_s(const MMSCoef *__restrict__ cf0, size_t cf_stride,
                                                           SloppyVecs v) {
     __shared__ float s_P[NS], s_a[NS], s_Q[NS][WIN], s_e[NS][WIN];
-    __shared__ int s_idx[NS];
+    __shared__ int s_idx[NS], s_used[WIN];
     __shared__ int s_n;
     dependent_begin();
     const int k = blockIdx.y;
     const MMSCoef *cf = (const MMSCoef *)((const char *)cf0 + k * cf_stride);
     if (threadIdx.x == 0) {
         int m = 0;
+        for (int l = 0; l < WIN; l++) s_used[l] = 0;
         for (int s = 0; s < v.nshift; s++)
             if (cf->touched[s]) {
                 s_idx[m] = s;
@@ -485,6 +486,7 @@ __global__ void __launch_bounds__(UPD_THREADS) k_window_s(const MMSCoef *__restr
                 for (int l = 0; l < WIN; l++) {
                     s_Q[m][l] = (float)cf->Q[s][l];
                     s_e[m][l] = (float)cf->e[s][l];
+                    if (s_Q[m][l] != 0.0f || s_e[m][l] != 0.0f) s_used[l] = 1;
                 }
                 m++;
             }
@@ -497,7 +499,8 @@ __global__ void __launch_bounds__(UPD_THREADS) k_window_s(const MMSCoef *__restr
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < v.n; i += (long)gridDim.x * blockDim.x) {
         float2 rv[WIN];
 #pragma unroll
-        for (int l = 0; l < WIN; l++) rv[l] = ring[l * v.n + i];
+        for (int l = 0; l < WIN; l++)  // slots past the solve's end hold no residual of this window
+            rv[l] = s_used[l] ? ring[l * v.n + i] : make_float2(0.0f, 0.0f);
         for (int q = 0; q < m; q++) {
             const size_t off = ((size_t)k * v.nshift + s_idx[q]) * v.n + i;
             const float2 pi = v.p0[off];
