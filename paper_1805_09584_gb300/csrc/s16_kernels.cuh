@@ -213,40 +213,40 @@ __global__ void __launch_bounds__(NT, MB) k_hop_even_s16(LatGeom g, int apbc, Si
     });
 }
 
-// Reduction partials: the FP32 sum over 8 threads (4 sites, both flavours; RP = 2: a right-hand side's 16 of the
-// warp) is added in FP64 to a shared slot per (sum, right-hand side, warp and lane).
+// Reduction partials: a site's 48 squares are added in FP32, the sites in FP64: two sites by a shuffle, then in a
+// shared slot per (right-hand side, sum, pair of sites).  Of two sums the second flavour's lanes do the second, so
+// that both take one FP64 instruction of each kind.  Against FP32 sums over 4 or 8 sites (four launches of an
+// iteration, 8 right-hand sides): 32^3x64 4.33 -> 4.23 ms, 24^3x48 1.32 -> 1.30 ms, 16^3x32 298 -> 307 us.
 template <bool DAG, int EPI, bool PF, int NT, int MB, int RP>
 __global__ void __launch_bounds__(NT, MB) k_hop_odd_s16(LatGeom g, int apbc, SiteTermF st, const int2 *__restrict__ links,
                                                         S16In psi_all, S16In te_all, S16Out out_all, S16EpiArgs ea,
                                                         int ntile, S16Batch bt) {
     constexpr bool SUMS = EPI == EPI_STORE_NORMS || EPI == EPI_MMS_R;
-    constexpr int NQ = EPI == EPI_STORE_NORMS ? 2 : 1, LANES = RP == 2 ? 1 : 4, SLOTS = NT / 32 * LANES;
+    constexpr int NQ = EPI == EPI_STORE_NORMS ? 2 : 1, SITES = Tile<NT, RP>::SITES, SLOTS = SITES / 2;
     __shared__ Tile<NT, RP> t;
-    __shared__ double part[SUMS ? NQ * TMND_MAX_BATCH * SLOTS : 1];
+    __shared__ double part[SUMS ? TMND_MAX_BATCH * NQ * SLOTS : 1];  // [nrhs][NQ][SLOTS]
     dependent_begin();
     if (ea.done && *ea.done) return;
     const Place<RP> pl;
     const int lane = threadIdx.x & 31, f = pl.f, Vh = g.Vh;
     if (SUMS)
-        for (int q = threadIdx.x; q < NQ * TMND_MAX_BATCH * SLOTS; q += NT) part[q] = 0.0;
+        for (int q = threadIdx.x; q < NQ * bt.nrhs * SLOTS; q += NT) part[q] = 0.0;
     int h = 0;
     auto tile = [&](int w) {
         __syncthreads();  // the previous tile is done with
-        load_tile<1, NT, RP>(g, apbc, links, w * Tile<NT, RP>::SITES, t);
-        h = w * Tile<NT, RP>::SITES + pl.i;
+        load_tile<1, NT, RP>(g, apbc, links, w * SITES, t);
+        h = w * SITES + pl.i;
         __syncthreads();
     };
     const float kp0 = (DAG ? -st.kp : st.kp) * (f == 0 ? 1.0f : -1.0f);
-    auto add = [&](float v, int q, int k, bool mine) {
-        v += __shfl_xor_sync(0xffffffffu, v, 16);
-        if (RP == 1) v += __shfl_xor_sync(0xffffffffu, v, 8);
-        v += __shfl_xor_sync(0xffffffffu, v, 4);
-        if (RP == 2) {
-            v += __shfl_xor_sync(0xffffffffu, v, 2);
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
-        }
-        const int l = RP == 2 ? lane & 7 : lane;  // RP 2: lane 0 holds the first right-hand side's sum, lane 8 the second's
-        if (mine && f == 0 && l < LANES) part[(q * TMND_MAX_BATCH + k) * SLOTS + (threadIdx.x >> 5) * LANES + l] += (double)v;
+    // lane bits: 4 flavour, 3 right-hand side (RP = 2) or site, 0..2 site; bit 2 makes the pairs
+    const int slot = (threadIdx.x >> 5) * (8 / RP) + (lane & 3) + (RP == 1 ? lane >> 1 & 4 : 0);
+    auto add = [&](float a, float b, int k, bool mine) {
+        a += __shfl_xor_sync(0xffffffffu, a, 16);
+        if (NQ == 2) b += __shfl_xor_sync(0xffffffffu, b, 16);
+        double d = (double)(NQ == 2 && f ? b : a);
+        d += __shfl_xor_sync(0xffffffffu, d, 4);
+        if (mine && !(lane & 4) && f < NQ) part[(NQ * k + f) * SLOTS + slot] += d;
     };
     walk<RP>(ntile, bt, tile, [&](int k0) {
         bool mine = true;
@@ -298,16 +298,20 @@ __global__ void __launch_bounds__(NT, MB) k_hop_odd_s16(LatGeom g, int apbc, Sit
             }
         }
         if (EPI != EPI_MMS_R) store_site(s16_at(out_all, k * bt.stride), f, hc, on, v);
-        if (SUMS) add(on ? s1 : 0.0f, 0, k, mine);
-        if (EPI == EPI_STORE_NORMS) add(on ? s2 : 0.0f, 1, k, mine);
+        if (SUMS) add(on ? s1 : 0.0f, on ? s2 : 0.0f, k, mine);
     });
     if (SUMS) {
         __syncthreads();
-        for (int w = threadIdx.x; w < NQ * bt.nrhs; w += NT) {
-            const int q = w / bt.nrhs, k = w - q * bt.nrhs;
+        constexpr int G = NT / 16;  // lanes per sum, 16 sums at a time
+        for (int w0 = 0; w0 < NQ * bt.nrhs; w0 += 16) {
+            const int w = w0 + threadIdx.x / G;
+            const bool valid = w < NQ * bt.nrhs;
             double s = 0.0;
-            for (int j = 0; j < SLOTS; j++) s += part[(q * TMND_MAX_BATCH + k) * SLOTS + j];
-            ea.part_out[(size_t)(NQ * k + q) * gridDim.x + blockIdx.x] = s;
+            if (valid)
+                for (int j = threadIdx.x % G; j < SLOTS; j += G) s += part[w * SLOTS + j];
+#pragma unroll
+            for (int off = G / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            if (valid && threadIdx.x % G == 0) ea.part_out[(size_t)w * gridDim.x + blockIdx.x] = s;
         }
     }
 }
