@@ -509,7 +509,6 @@ __global__ void __launch_bounds__(256) k_fx_to_f32(int Vh, double a, FxIn in, fl
 __global__ void __launch_bounds__(128) k_fx_pupdate(int Vh, const int *__restrict__ skip,
                                                     const double *__restrict__ beta_p,
                                                     const double2 *__restrict__ r, FxOut p) {
-    dependent_begin();
     if (*skip) return;
     const double beta = *beta_p;
     const int lane = threadIdx.x & 31, f = lane >> 4;
@@ -635,7 +634,7 @@ void launch_fx_to_f32(const Geom &g, double a, FxIn in, float2 *out, cudaStream_
 void launch_fx_pupdate(const Geom &g, const int *skip, const double *beta, const double2 *r, FxOut p,
                        cudaStream_t s) {
     const int groups = (g.Vh + 15) / 16;
-    launch_dependent(k_fx_pupdate, dim3((groups + 3) / 4), 128, s, g.Vh, skip, beta, r, p);
+    k_fx_pupdate<<<(groups + 3) / 4, 128, 0, s>>>(g.Vh, skip, beta, r, p);
 }
 
 void launch_fx_pack_links(const Geom &g, const double2 *canon, int4 *out, cudaStream_t s) {

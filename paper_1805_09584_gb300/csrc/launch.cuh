@@ -2,7 +2,8 @@
 // launch): a chain of kernels of a few microseconds each, as in an operator application on a small lattice,
 // then does not pay a launch latency per link (FP64 Qhat^2 + sigma, five kernels: 4^4 31 -> 23 us, 16^3x32
 // 249 -> 240 us).  Not while the stream is being captured: between the nodes of a graph the plain
-// dependency is the faster one (FP64 solve on 8^3x16 9.2 ms, 11.8 ms with programmatic edges).
+// dependency is the faster one (FP64 solve on 8^3x16 9.2 ms, 11.8 ms with programmatic edges), so kernels that run
+// in the solvers' graphs only are launched plainly.
 //
 // A kernel started with launch_dependent() may begin as soon as every block of its predecessor has begun and
 // there is room.  It calls dependent_begin() first: that lets its own successor be set up, and waits until

@@ -44,7 +44,6 @@
 #include <vector>
 
 #include "fx_sum.cuh"
-#include "launch.cuh"
 
 namespace {
 
@@ -237,7 +236,6 @@ __global__ void __launch_bounds__(SCAL_THREADS) k_scalars(MMSState *st, MMSCoef 
                                                           const double *__restrict__ part_rr, MMSConst c, int j,
                                                           double *hist, int hist_cap) {
     __shared__ double red[40];
-    dependent_begin();
     scalars_step(st, cf, nb_hop, part_rr, c, j, hist, hist_cap, red);
 }
 
@@ -252,7 +250,6 @@ __global__ void __launch_bounds__(SCAL_THREADS) k_scalars_b(MMSState *st, MMSCoe
     __shared__ double red[40];
     const int k = blockIdx.x;
     const MMSConst ck = const_of(c, bc, k);
-    dependent_begin();
     const bool end = scalars_step((MMSState *)((char *)st + k * st_stride), (MMSCoef *)((char *)cf + k * cf_stride),
                                   nb_hop, part_rr + (size_t)k * nb_hop, ck, j, k == 0 ? hist : nullptr, hist_cap, red);
     if (end && threadIdx.x == 0 && atomicAdd(&done_all[1], 1) + 1 == (int)gridDim.x) done_all[0] = 1;
@@ -265,7 +262,6 @@ __global__ void k_alpha(MMSState *st, size_t st_stride, const double *__restrict
                         BatchConst bc) {
     __shared__ double red[40];
     const int k = blockIdx.x;
-    dependent_begin();
     st = (MMSState *)((char *)st + k * st_stride);
     if (st->done) return;
     const double *part = part_norm + (size_t)2 * k * nb_hop;
@@ -296,7 +292,6 @@ __global__ void __launch_bounds__(UPD_THREADS, WINDOW_BLOCKS) k_window(long n, c
     __shared__ int s_e[NS][2], s_ep[NS][2];   // exponents of the sums' units: over l, p_i's term
     __shared__ int s_idx[NS], s_ok[NS][2], s_used[WIN];
     __shared__ int s_n;
-    dependent_begin();
     if (threadIdx.x < WIN) s_used[threadIdx.x] = 0;
     if (threadIdx.x < 32) {
         static_assert(NS <= 32, "a lane per shift");
@@ -445,7 +440,6 @@ __global__ void k_init_s(int Vh, SloppyVecs v, double *__restrict__ part) {
 
 // p = r' + beta p for right-hand side blockIdx.y (slot j of its ring), p stored in 16 bits
 __global__ void k_pupdate_s(int Vh, const MMSCoef *__restrict__ cf0, size_t cf_stride, SloppyVecs v, int j) {
-    dependent_begin();
     const int k = blockIdx.y;
     const MMSCoef *cf = (const MMSCoef *)((const char *)cf0 + k * cf_stride);
     if (cf->skip) return;
@@ -472,7 +466,6 @@ __global__ void __launch_bounds__(UPD_THREADS) k_window_s(const MMSCoef *__restr
     __shared__ float s_P[NS], s_a[NS], s_Q[NS][WIN], s_e[NS][WIN];
     __shared__ int s_idx[NS], s_used[WIN];
     __shared__ int s_n;
-    dependent_begin();
     const int k = blockIdx.y;
     const MMSCoef *cf = (const MMSCoef *)((const char *)cf0 + k * cf_stride);
     if (threadIdx.x == 0) {
@@ -758,7 +751,7 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
         e1.done = &st->done;
         launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(p), te, false, &st->done, s);
         launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(p), fx_in(te), false, FX_STORE_NORMS, e1, s);
-        launch_dependent(k_alpha, dim3(1), 256, s, st, 0, part_norm, nb_hop, c.sigma0, BatchConst());
+        k_alpha<<<1, 256, 0, s>>>(st, 0, part_norm, nb_hop, c.sigma0, BatchConst());
         launch_fx_even(g->geom, g->fx, g->links_fx, fx_in(y), te, true, &st->done, s);
         FxOdd e2 = {};
         e2.sigma = c.sigma0;
@@ -770,9 +763,9 @@ static tmnd_status mms_one_rhs(tmnd_gauge *g, const double2 *b, double2 *const *
         e2.done = &st->done;
         launch_fx_odd(g->geom, g->fx, g->links_fx, fx_in(y), fx_in(te), true, FX_MMS_R, e2, s);
         mark(1);
-        launch_dependent(k_scalars, dim3(1), SCAL_THREADS, s, st, cf, nb_hop, part_rr, c, j, hist, hist_cap);
+        k_scalars<<<1, SCAL_THREADS, 0, s>>>(st, cf, nb_hop, part_rr, c, j, hist, hist_cap);
         launch_fx_pupdate(g->geom, &cf->skip, &cf->beta, slot[j], p, s);
-        if (j == WIN - 1) launch_dependent(k_window, dim3(nb_win), UPD_THREADS, s, n, cf, ring, ptrs, nshift);
+        if (j == WIN - 1) k_window<<<nb_win, UPD_THREADS, 0, s>>>(n, cf, ring, ptrs, nshift);
         mark(2);
     };
     LoopOut lo;
@@ -999,7 +992,7 @@ static tmnd_status mms_sloppy(tmnd_gauge *g, const MixedWork &m, const double *s
         e1.done = done_all;
         launch_hop_even_s16(g->geom, g->stf, g->links_s16, p16i, te16, false, done_all, s, bt);
         launch_hop_odd_s16(g->geom, g->stf, g->links_s16, p16i, te16i, y16, false, EPI_STORE_NORMS, e1, s, bt);
-        launch_dependent(k_alpha, dim3(R), 256, s, st, st_stride, part_norm, nb_hop, c.sigma0, bc);
+        k_alpha<<<R, 256, 0, s>>>(st, st_stride, part_norm, nb_hop, c.sigma0, bc);
         launch_hop_even_s16(g->geom, g->stf, g->links_s16, y16i, te16, true, done_all, s, bt);
         S16EpiArgs e2 = {};
         e2.sigma = c.sigma0;
@@ -1015,10 +1008,10 @@ static tmnd_status mms_sloppy(tmnd_gauge *g, const MixedWork &m, const double *s
         for (int q = 0; q < R && bc.on; q++) e2.sigma_k[q] = bc.sigma0[q];
         launch_hop_odd_s16(g->geom, g->stf, g->links_s16, y16i, te16i, S16Out{}, true, EPI_MMS_R, e2, s, bt);
         mark(1);
-        launch_dependent(k_scalars_b, dim3(R), SCAL_THREADS, s, st, cf, st_stride, cf_stride, nb_hop, part_rr, c, bc, j,
-                         hist, hist_cap, done_all);
-        launch_dependent(k_pupdate_s, dim3(nb_site, R), 128, s, Vh, cf, cf_stride, v, j);
-        if (j == WIN - 1) launch_dependent(k_window_s, dim3(nb_str, R), UPD_THREADS, s, cf, cf_stride, v);
+        k_scalars_b<<<R, SCAL_THREADS, 0, s>>>(st, cf, st_stride, cf_stride, nb_hop, part_rr, c, bc, j, hist, hist_cap,
+                                               done_all);
+        k_pupdate_s<<<dim3(nb_site, R), 128, 0, s>>>(Vh, cf, cf_stride, v, j);
+        if (j == WIN - 1) k_window_s<<<dim3(nb_str, R), UPD_THREADS, 0, s>>>(cf, cf_stride, v);
         mark(2);
     };
     tmnd_status ls = run_graph_loop(s, done_all, maxiter, check_every, profile, body, lo);
