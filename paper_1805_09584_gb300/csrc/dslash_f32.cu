@@ -42,7 +42,7 @@ __device__ __forceinline__ float2 Bdag(const float2 v[2][3], int s, int c) {
 // U_mu(x), -1 backward with U_mu(x-mu)^+) into acc[spin][colour]; sg = -1 across the antiperiodic boundary.
 // G5IN: the input field is gamma_5 psi (lower spins negated).
 template <int MU, int DIR, bool G5IN>
-__device__ __forceinline__ void hop_dir(const float2 *__restrict__ in, const float2 *__restrict__ U, int Vh, float sg,
+__device__ __forceinline__ void hop_dir(const float2 *in, const float2 *__restrict__ U, int Vh, float sg,
                                         float2 acc[4][3]) {
     // sign of the B psi_lo term in chi: forward -, backward +; gamma_5 on input flips it
     constexpr bool plus = (DIR < 0) != G5IN;
@@ -51,8 +51,8 @@ __device__ __forceinline__ void hop_dir(const float2 *__restrict__ in, const flo
     for (int s = 0; s < 2; s++)
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-            up[s][c] = __ldg(&in[(s * 3 + c) * Vh]);
-            lo[s][c] = __ldg(&in[((s + 2) * 3 + c) * Vh]);
+            up[s][c] = in[(s * 3 + c) * Vh];
+            lo[s][c] = in[((s + 2) * 3 + c) * Vh];
         }
     float2 chi[2][3];
 #pragma unroll
@@ -88,7 +88,7 @@ __device__ __forceinline__ void hop_dir(const float2 *__restrict__ in, const flo
 // H applied at output site h of parity P to one flavour; in: that flavour's planes on parity 1 - P.
 template <int P, bool G5IN>
 __device__ __forceinline__ void hop_all(const LatGeom &g, int apbc, const float2 *__restrict__ links,
-                                        const float2 *__restrict__ in, int h, float2 acc[4][3]) {
+                                        const float2 *in, int h, float2 acc[4][3]) {
     const int Vh = g.Vh;
     const float2 *Lp = links + (size_t)P * 4 * 9 * Vh;        // links based at parity P sites
     const float2 *Lq = links + (size_t)(1 - P) * 4 * 9 * Vh;  // links based at parity 1-P sites
@@ -136,7 +136,7 @@ SiteTerm32 site32(const SiteTerm &st, bool dag) {
 template <bool DAG>
 __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_even_f32(LatGeom g, int apbc, SiteTerm32 st,
                                                                      const float2 *__restrict__ links,
-                                                                     const float2 *__restrict__ psi,
+                                                                     const float2 *psi,
                                                                      float2 *__restrict__ out) {
     dependent_begin();
     const int lane = threadIdx.x & 31, f = lane >> 4, Vh = g.Vh;
@@ -162,8 +162,8 @@ __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_even_f32(LatGeom g,
 template <bool DAG, int EPI>
 __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_odd_f32(LatGeom g, int apbc, SiteTerm32 st,
                                                                     const float2 *__restrict__ links,
-                                                                    const float2 *__restrict__ psi,
-                                                                    const float2 *__restrict__ te,
+                                                                    const float2 *psi,
+                                                                    const float2 *te,
                                                                     float2 *__restrict__ out, HopEpiArgsF ea) {
     dependent_begin();
     const int lane = threadIdx.x & 31, f = lane >> 4, Vh = g.Vh;
@@ -175,6 +175,13 @@ __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_odd_f32(LatGeom g, 
     const float sigma = EPI == EPI_SHIFT ? ea.sigma[ea.per_rhs ? blockIdx.y : 0] : 0.0f;
     const float2 *own = psi + off + h, *oth = psi + (size_t)blockIdx.y * NCOMP * Vh + (size_t)(1 - f) * 12 * Vh + h;
     float2 *o = out + off + h;
+    float2 po[12], qo[12], ao[12];  // all loads before the first store, which plain loads may not pass
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+        po[k] = own[k * Vh];
+        qo[k] = oth[k * Vh];
+        if (EPI == EPI_SHIFT) ao[k] = ea.aux[off + h + (size_t)k * Vh];
+    }
 #pragma unroll
     for (int s = 0; s < 4; s++) {
         const float b = (f == 0) == (s < 2) ? st.kp : -st.kp;
@@ -182,12 +189,12 @@ __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_odd_f32(LatGeom g, 
         const bool hopneg = DAG && s >= 2;
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-            const float2 p = __ldg(&own[(s * 3 + c) * Vh]), q = __ldg(&oth[(s * 3 + c) * Vh]);
+            const float2 p = po[s * 3 + c], q = qo[s * 3 + c];
             const float2 hp = hopneg ? cneg(acc[s][c]) : acc[s][c];
             // A = [[1 + i kp g, -kpp],[-kpp, 1 - i kp g]]
             float2 y = make_float2(fmaf(-b, p.y, fmaf(-st.kpp, q.x, p.x - hp.x)), fmaf(b, p.x, fmaf(-st.kpp, q.y, p.y - hp.y)));
             if (EPI == EPI_SHIFT) {
-                const float2 a = __ldg(&ea.aux[off + h + (size_t)(s * 3 + c) * Vh]);
+                const float2 a = ao[s * 3 + c];
                 y = make_float2(fmaf(sigma, a.x, y.x), fmaf(sigma, a.y, y.y));
             }
             o[(s * 3 + c) * Vh] = y;
@@ -199,7 +206,7 @@ __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_odd_f32(LatGeom g, 
 // + i s gamma_5 tau_1 x.  NF = 1: one flavour, D_TM(+mu) (kpp and s ignored), 32 sites per warp.
 template <int NF, int P>
 __device__ __forceinline__ void dnd_sites(const LatGeom &g, int apbc, float kappa, float kp, float kpp, float so,
-                                          const float2 *__restrict__ links, const float2 *__restrict__ in,
+                                          const float2 *__restrict__ links, const float2 *in,
                                           float2 *__restrict__ out) {
     const int lane = threadIdx.x & 31, f = NF == 2 ? lane >> 4 : 0, Vh = g.Vh;
     constexpr int SITES = NF == 2 ? 16 : 32;
@@ -210,16 +217,22 @@ __device__ __forceinline__ void dnd_sites(const LatGeom &g, int apbc, float kapp
     hop_all<P, false>(g, apbc, links, in + (1 - P) * n + (size_t)f * 12 * Vh, h, acc);
     const float2 *own = in + P * n + (size_t)f * 12 * Vh + h, *oth = in + P * n + (size_t)(NF - 1 - f) * 12 * Vh + h;
     float2 *o = out + P * n + (size_t)f * 12 * Vh + h;
+    float2 po[12], qo[12];
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+        po[k] = own[k * Vh];
+        if (NF == 2) qo[k] = oth[k * Vh];
+    }
 #pragma unroll
     for (int s = 0; s < 4; s++) {
         const float g5 = s < 2 ? 1.0f : -1.0f;
         const float b = f == 0 ? kp * g5 : -kp * g5, e = P == 1 ? so * g5 : 0.0f;
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-            const float2 p = __ldg(&own[(s * 3 + c) * Vh]);
+            const float2 p = po[s * 3 + c];
             float2 y = make_float2(fmaf(-b, p.y, fmaf(-kappa, acc[s][c].x, p.x)), fmaf(b, p.x, fmaf(-kappa, acc[s][c].y, p.y)));
             if (NF == 2) {
-                const float2 q = __ldg(&oth[(s * 3 + c) * Vh]);
+                const float2 q = qo[s * 3 + c];
                 y = make_float2(fmaf(-kpp, q.x, fmaf(-e, q.y, y.x)), fmaf(-kpp, q.y, fmaf(e, q.x, y.y)));
             }
             o[(s * 3 + c) * Vh] = y;
@@ -229,7 +242,7 @@ __device__ __forceinline__ void dnd_sites(const LatGeom &g, int apbc, float kapp
 template <int NF>
 __global__ void __launch_bounds__(F32_THREADS, F32_BLOCKS) k_dnd(LatGeom g, int apbc, float kappa, float kp, float kpp,
                                                                 float so, const float2 *__restrict__ links,
-                                                                const float2 *__restrict__ in, float2 *__restrict__ out) {
+                                                                const float2 *in, float2 *__restrict__ out) {
     dependent_begin();
     if (blockIdx.y == 0) dnd_sites<NF, 0>(g, apbc, kappa, kp, kpp, so, links, in, out);
     else dnd_sites<NF, 1>(g, apbc, kappa, kp, kpp, so, links, in, out);

@@ -33,7 +33,7 @@ namespace {
 // chi = up -+ B lo, or of its complex conjugate for the backward hop (see hop_run).  G5IN: the input is
 // gamma_5 psi.
 template <int MU, int DIR, bool G5IN>
-__device__ __forceinline__ void project(const int4 *__restrict__ in, int ch[2][3][2], int cl[2][3][2]) {
+__device__ __forceinline__ void project(const int4 *in, int ch[2][3][2], int cl[2][3][2]) {
     constexpr bool plus = (DIR < 0) != G5IN;   // sign of B psi_lo in chi
     constexpr bool swap = MU == 1 || MU == 2;  // B connects spin s with lower spin 1 - s
     constexpr bool imag = MU == 1 || MU == 3;
@@ -45,8 +45,8 @@ __device__ __forceinline__ void project(const int4 *__restrict__ in, int ch[2][3
         const bool sub = neg == plus;  // chi = up -+ (lo or i lo), i lo = (-lo.im, lo.re)
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-            const int4 a = __ldg(&in[(s * 3 + c) * FX_RUN]);
-            const int4 b = __ldg(&in[((2 + sl) * 3 + c) * FX_RUN]);
+            const int4 a = in[(s * 3 + c) * FX_RUN];
+            const int4 b = in[((2 + sl) * 3 + c) * FX_RUN];
             ch[s][c][0] = imag ? (sub ? a.x + b.z : a.x - b.z) : (sub ? a.x - b.x : a.x + b.x);
             cl[s][c][0] = imag ? (sub ? a.y + b.w : a.y - b.w) : (sub ? a.y - b.y : a.y + b.y);
             const int ih = imag ? (sub ? a.z - b.x : a.z + b.x) : (sub ? a.z - b.z : a.z + b.z);
@@ -174,8 +174,8 @@ __device__ __forceinline__ int hop_sum(const FxShared &sm, int spin, long long v
 // takes direction mu, then adds up the four directions of spin mu: v 2^(e - 56), |v| <= 2^61.3, with the
 // flavour of the lane's half.  Returns e, the largest exponent among the neighbours.
 template <int P, bool G5IN>
-__device__ __forceinline__ int hop_run(const LatGeom &g, const int4 *__restrict__ links, const int4 *__restrict__ in,
-                                       const int *__restrict__ ex, int h, FxShared &sm, long long v[3][2]) {
+__device__ __forceinline__ int hop_run(const LatGeom &g, const int4 *__restrict__ links, const int4 *in,
+                                       const int *ex, int h, FxShared &sm, long long v[3][2]) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int nb[2];
     switch (w) {
@@ -184,7 +184,7 @@ __device__ __forceinline__ int hop_run(const LatGeom &g, const int4 *__restrict_
         case 2: neighbours<2, P>(g, h, nb[0], nb[1]); break;
         default: neighbours<3, P>(g, h, nb[0], nb[1]);
     }
-    const int ef = __ldg(&ex[nb[0]]), eb = __ldg(&ex[nb[1]]), em = max(ef, eb);
+    const int ef = ex[nb[0]], eb = ex[nb[1]], em = max(ef, eb);
     const size_t mu_stride = 9 * fx_sites(g.Vh);
     const int4 *qf = in + fx_at(nb[0], 24), *qb = in + fx_at(nb[1], 24);
     const int4 *uf = links + ((size_t)P * 4 + w) * mu_stride + fx_at(h, 9);
@@ -279,7 +279,7 @@ __device__ __forceinline__ void mac(int2 c, int h, int l, long long &x, long lon
 // even sites: t_e = kappa^2 A^-1 H psi  (DAG: kappa^2 A(-mu)^-1 H gamma_5 psi)
 template <bool DAG>
 __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_even(LatGeom g, FxSite st, const int4 *__restrict__ links,
-                                                                   FxIn psi, FxOut out, const int *__restrict__ done,
+                                                                   FxIn psi, FxOut out, const int *done,
                                                                    int nrun, FxBatch bt) {
     __shared__ FxShared sm;
     dependent_begin();
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_odd(LatGeom g, FxS
         const int ez = ep + st.fwd_e;
         int em = max(ez - 4, eh), es = FX_ZERO;
         if (EPI == FX_MMS_R) {
-            es = __ldg(&ea.p.e[h]) + ea.sig_e;
+            es = ea.p.e[h] + ea.sig_e;
             em = max(em, es - 4);
         }
         const int sa = min(em - eh, 63), sz = min(em - (ez - 4), 63), ss = min(em - (es - 4), 63);
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_odd(LatGeom g, FxS
             const int4 p = psi.q[at + c * FX_RUN];
             const int4 o = psi.q[ot + c * FX_RUN];
             int4 pp;
-            if (EPI == FX_MMS_R) pp = __ldg(&ea.p.q[at + c * FX_RUN]);
+            if (EPI == FX_MMS_R) pp = ea.p.q[at + c * FX_RUN];
             const int ph[2] = {p.x, p.z}, pl[2] = {p.y, p.w};
             const int oh[2] = {o.x, o.z}, ol[2] = {o.y, o.w};
 #pragma unroll
@@ -423,6 +423,11 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_odd(LatGeom g, FxS
         } else {
             const FxScale sc = fx_scale(em, em - 56);
             const double al = EPI == FX_MMS_R ? -alpha * sc.s1 : 0.0;
+            double2 aux[3];  // loaded before the first store, which plain loads may not pass
+            if (EPI == FX_F64_SHIFT || EPI == FX_RESID) {
+#pragma unroll
+                for (int c = 0; c < 3; c++) aux[c] = ea.aux64[off64 + (size_t)(f * 12 + s * 3 + c) * Vh + h];
+            }
 #pragma unroll
             for (int c = 0; c < 3; c++) {
                 const size_t i = (size_t)(f * 12 + s * 3 + c) * Vh + h;
@@ -436,11 +441,11 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_odd(LatGeom g, FxS
                     const double sg = s < 2 ? 1.0 : -1.0;
                     ea.out64[off64 + j] = make_double2(sg * fx_to_double(vr, sc), sg * fx_to_double(vi, sc));
                 } else if (EPI == FX_F64_SHIFT) {
-                    const double2 a = __ldg(&ea.aux64[off64 + i]);
+                    const double2 a = aux[c];
                     ea.out64[off64 + i] = make_double2(fma(ea.sigma, a.x, fx_to_double(vr, sc)),
                                                        fma(ea.sigma, a.y, fx_to_double(vi, sc)));
                 } else if (EPI == FX_RESID) {
-                    const double2 a = __ldg(&ea.aux64[i]), bv = __ldg(&ea.b64[i]);
+                    const double2 a = aux[c], bv = ea.b64[i];
                     const double2 r1 = make_double2(bv.x - fma(ea.sigma, a.x, fx_to_double(vr, sc)),
                                                     bv.y - fma(ea.sigma, a.y, fx_to_double(vi, sc)));
                     ea.r[i] = r1;
@@ -474,7 +479,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_BLOCKS) k_fx_odd(LatGeom g, FxS
 }
 
 // FP64 planes -> digits
-__global__ void __launch_bounds__(128) k_fx_from_f64(int Vh, const double2 *__restrict__ in, FxOut out, FxBatch bt) {
+__global__ void __launch_bounds__(128) k_fx_from_f64(int Vh, const double2 *in, FxOut out, FxBatch bt) {
     dependent_begin();
     in += blockIdx.y * bt.n64;
     out = fx_next(out, blockIdx.y * bt.stride);
@@ -483,7 +488,7 @@ __global__ void __launch_bounds__(128) k_fx_from_f64(int Vh, const double2 *__re
     const int hh = gr * 16 + (lane & 15), h = min(hh, Vh - 1);
     double2 v[12];
 #pragma unroll
-    for (int c = 0; c < 12; c++) v[c] = __ldg(&in[(size_t)(f * 12 + c) * Vh + h]);
+    for (int c = 0; c < 12; c++) v[c] = in[(size_t)(f * 12 + c) * Vh + h];
     int4 q[12];
     int e;
     fx_from_doubles(v, q, e);

@@ -43,8 +43,8 @@ __device__ __forceinline__ int word(const Raw &r, int k) {
 __device__ __forceinline__ void load_raw(const S16In &in, int f, int h, Raw &r) {
     const int4 *q = in.q + s16_qi(f * 3, h);
 #pragma unroll
-    for (int j = 0; j < 3; j++) r.q[j] = __ldg(q + j * S16_BLOCK_SITES);
-    r.nrm = __ldg(&in.nrm[s16_ni(h)]);
+    for (int j = 0; j < 3; j++) r.q[j] = q[j * S16_BLOCK_SITES];
+    r.nrm = in.nrm[s16_ni(h)];
 }
 
 // (u.x + SX l.x, u.y + SY l.y) for biased floats u, l (exact integer results)

@@ -181,7 +181,7 @@ struct Place {
 
 template <bool DAG, bool PF, int NT, int MB, int RP>
 __global__ void __launch_bounds__(NT, MB) k_hop_even_s16(LatGeom g, int apbc, SiteTermF st, const int2 *__restrict__ links,
-                                                         S16In in, S16Out out, const int *__restrict__ done, int ntile,
+                                                         S16In in, S16Out out, const int *done, int ntile,
                                                          S16Batch bt) {
     __shared__ Tile<NT, RP> t;
     dependent_begin();
