@@ -186,7 +186,8 @@ tmnd_status tm_nd_apply_noalloc(const tmnd_gauge *g, void *out, const void *in, 
 /* Launch-shape autotuner of the sloppy (16-bit) stencil.  Its kernels run in
  * TMND_S16_SHAPES launch variants: 4 compiled shapes (threads per block x resident blocks
  * per SM the register budget is cut for x next-direction prefetch; shape 0 takes one right-hand
- * side per pass over a block's tile of sites, the others two) x 4 loop orders (0: every
+ * side per pass over a block's tile of sites, 1 and 2 take two; shape 3 has a thread per site and no
+ * tiles, for one right-hand side; its orders 1 and 3 are 0 and 2) x 4 loop orders (0: every
  * block walks its own tiles, all right-hand sides of a tile in turn; 1: its tiles
  * once per right-hand side; 2: all blocks sweep the lattice together by grid stride, all
  * right-hand sides of a tile in turn; 3: grid stride over (tile, right-hand side) items);

@@ -1,5 +1,5 @@
 // Sloppy stencil, host side: dispatch over the compiled launch shapes (kernels in
-// s16_kernels.cuh, one translation unit per shape: dslash_s16_v*.cu) and the autotuner
+// s16_kernels.cuh and s16_site.cuh, one translation unit per shape: dslash_s16_v*.cu) and the autotuner
 // that picks a launch variant per (lattice, right-hand sides per launch).
 #include <array>
 #include <map>
@@ -31,6 +31,7 @@ constexpr int NCOMPILED = sizeof(kShapes) / sizeof(kShapes[0]);
 // block walks its own tiles of sites, all right-hand sides of a tile in turn; 1 = the same
 // tiles once per right-hand side; 2 = all blocks sweep the lattice together (grid stride),
 // all right-hand sides of a tile in turn; 3 = grid stride over (tile, right-hand side) items
+// (s16_site.cuh: 1 is 0, 3 is 2, with sites for tiles)
 constexpr int NORDERS = 4;
 constexpr int NSHAPES = NORDERS * NCOMPILED;
 static_assert(NSHAPES == TMND_S16_SHAPES, "variant count of include/tmnd.h");
@@ -89,7 +90,7 @@ std::array<int, 6> tune_key(const Geom &g, int nrhs) {
 int hop_blocks_s16(const Geom &g, int shape) {
     if (shape < 0 || shape >= NSHAPES) shape = 0;
     const ShapeDesc &d = kShapes[shape % NCOMPILED];
-    const int sites = d.threads / (2 * d.rp);  // per tile
+    const int sites = d.rp ? d.threads / (2 * d.rp) : d.threads;  // per tile
     const int cap = sm_count() * per_sm(shape);
     const int want = (g.Vh + sites - 1) / sites;
     return want < cap ? want : cap;

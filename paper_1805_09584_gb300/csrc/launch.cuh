@@ -18,22 +18,28 @@
 
 #include <cuda_runtime.h>
 
-// overlap = false: a plain launch
+// overlap = false: a plain launch; smem: bytes of dynamic shared memory
 template <typename... P, typename... A>
-inline void launch_dependent_if(bool overlap, void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s,
-                                A &&...args) {
+inline void launch_dependent_smem(bool overlap, void (*kernel)(P...), dim3 grid, unsigned block, size_t smem,
+                                  cudaStream_t s, A &&...args) {
     cudaLaunchAttribute attr = {};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t c = {};
     c.gridDim = grid;
     c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
     c.stream = s;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(s, &capture);
     c.attrs = &attr;
     c.numAttrs = overlap && capture == cudaStreamCaptureStatusNone ? 1 : 0;
     cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);  // an error stays pending for the caller's check
+}
+template <typename... P, typename... A>
+inline void launch_dependent_if(bool overlap, void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s,
+                                A &&...args) {
+    launch_dependent_smem(overlap, kernel, grid, block, 0, s, static_cast<A &&>(args)...);
 }
 template <typename... P, typename... A>
 inline void launch_dependent(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, A &&...args) {

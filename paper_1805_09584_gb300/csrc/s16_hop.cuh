@@ -46,6 +46,12 @@ __device__ __forceinline__ void load_raw(const S16In &in, int f, int h, Raw &r) 
     for (int j = 0; j < 3; j++) r.q[j] = q[j * S16_BLOCK_SITES];
     r.nrm = in.nrm[s16_ni(h)];
 }
+__device__ __forceinline__ void load_raw2(const S16In &in, int h, Raw r[2]) {  // both flavours
+    const int4 *q = in.q + s16_qi(0, h);
+#pragma unroll
+    for (int j = 0; j < 6; j++) r[j / 3].q[j % 3] = q[j * S16_BLOCK_SITES];
+    r[0].nrm = r[1].nrm = in.nrm[s16_ni(h)];
+}
 
 // (u.x + SX l.x, u.y + SY l.y) for biased floats u, l (exact integer results)
 template <int SX, int SY>
@@ -55,10 +61,8 @@ __device__ __forceinline__ f2 comb(f2 u, f2 l) {
     return SX > 0 && SY > 0 ? add2(v, l) : fma2(l, make_float2((float)SX, (float)SY), v);
 }
 
-// Decode a link (rows 0 and 1, scale 32767) and rebuild row 2 = conj(row 0 x row 1) (det U = 1) as
-// integer-valued floats at that scale, times sg (+-1).  u: 9 complex numbers, row-major.
-__device__ __forceinline__ void decode_link(const int2 *__restrict__ L, int h, float sg, f2 u[9]) {
-    int wv[6];
+// A link's words: rows 0 and 1, scale 32767
+__device__ __forceinline__ void load_link(const int2 *__restrict__ L, int h, int wv[6]) {
 #pragma unroll
     for (int j = 0; j < 3; j++) {
         int2 w;
@@ -66,6 +70,10 @@ __device__ __forceinline__ void decode_link(const int2 *__restrict__ L, int h, f
         wv[2 * j] = w.x;
         wv[2 * j + 1] = w.y;
     }
+}
+// Decode a link and rebuild row 2 = conj(row 0 x row 1) (det U = 1) as integer-valued floats at that scale,
+// times sg (+-1).  u: 9 complex numbers, row-major.
+__device__ __forceinline__ void decode_link(const int wv[6], float sg, f2 u[9]) {
 #pragma unroll
     for (int k = 0; k < 6; k++) u[k] = make_float2(s16_lo(wv[k]), s16_hi(wv[k]));
 #pragma unroll

@@ -24,12 +24,11 @@
 // instead of 16; with RP = 1 that traffic keeps the L1 data pipe 68 % busy): 7 % faster at 16^3x32 with 8 right-hand
 // sides, 2 % slower at 24^3x48, useless for one.
 //
-// The form before this one had one thread per site for both flavours, which decoded and rebuilt the links
-// for every right-hand side (60 of 225 instructions per direction) at 168 registers, 12 warps per SM, and was
-// bound by issue and latency together.  Four launches of Qhat^2 + sigma, before and now: 24^3x48 1 right-hand
-// side 0.22 -> 0.23 ms, 8 1.47 -> 1.29 ms; 16^3x32 8 0.39 -> 0.29 ms; an iteration of the multi-shift solver at
-// 24^3x48 with 8 (the residual update's FP32 planes loaded all at once) 1.9 -> 1.33 ms.  Now: FP32 pipe 53 %,
-// issue 55 %, 17 warps per SM.
+// One thread per site for both flavours (s16_site.cuh) decodes and rebuilds the links for every right-hand side (60
+// of 225 instructions per direction) at 168 registers, 12 warps per SM.  Four launches of Qhat^2 + sigma, that form
+// and this one: 24^3x48 8 right-hand sides 1.47 -> 1.25 ms; 16^3x32 8 0.35 -> 0.28 ms; an iteration of the
+// multi-shift solver at 24^3x48 with 8 (the residual update's FP32 planes loaded all at once) 1.60 -> 1.30 ms.  Here:
+// FP32 pipe 53 %, issue 55 %, 17 warps per SM.
 //
 // This header holds the kernel templates; each compiled launch shape is instantiated
 // in a translation unit of its own (dslash_s16_v*.cu, built in parallel) through
@@ -43,9 +42,10 @@
 namespace {
 
 // Launch shapes the kernels are compiled in: threads per block, resident blocks per SM the register budget is
-// cut for, next-direction prefetch, right-hand sides per pass.  The autotuner times each on the GPU per
-// (lattice, right-hand sides per launch) and keeps the fastest; shape 0 is the default.
-#define TMND_S16_SHAPE_LIST(X) X(0, 128, 4, true, 1) X(1, 128, 5, true, 2) X(2, 64, 8, true, 2) X(3, 64, 7, true, 2)
+// cut for, next-direction prefetch, right-hand sides per pass (0: the form of s16_site.cuh, a site per thread).  The
+// autotuner times each on the GPU per (lattice, right-hand sides per launch) and keeps the fastest; shape 0 is the
+// default.
+#define TMND_S16_SHAPE_LIST(X) X(0, 128, 4, true, 1) X(1, 128, 5, true, 2) X(2, 64, 8, true, 2) X(3, 128, 3, true, 0)
 
 template <int NT, int RP>
 struct Tile {
@@ -83,9 +83,12 @@ __device__ __forceinline__ void load_tile(const LatGeom &g, int apbc, const int2
         t.nb[2 * mu][i] = hf;
         t.nb[2 * mu + 1][i] = hb;
         f2 u[9];
-        decode_link(Lp + mu * stride, h, sf, u);
+        int wv[6];
+        load_link(Lp + mu * stride, h, wv);
+        decode_link(wv, sf, u);
         t.links.put(2 * mu, i, u);
-        decode_link(Lq + mu * stride, hb, sb, u);
+        load_link(Lq + mu * stride, hb, wv);
+        decode_link(wv, sb, u);
         t.links.put(2 * mu + 1, i, u);
     }
 }
