@@ -7,7 +7,7 @@
 
 #include "s16_kernels.cuh"
 
-#define TMND_S16_DECL(I, T, B, P, R)                                                                               \
+#define TMND_S16_DECL(I, T, B, R)                                                                                  \
     int s16_per_sm_##I();                                                                                       \
     void s16_even_##I(const Geom &g, const SiteTermF &st, const int2 *links, S16In in, S16Out out, bool dag,   \
                       const int *done, cudaStream_t s, const S16Batch &bt, int nb);                             \
@@ -19,10 +19,10 @@ TMND_S16_SHAPE_LIST(TMND_S16_DECL)
 namespace {
 
 struct ShapeDesc {
-    int threads, minb, pf, rp;
+    int threads, minb, rp;
 };
 constexpr ShapeDesc kShapes[] = {
-#define TMND_S16_DESC(I, T, B, P, R) {T, B, P, R},
+#define TMND_S16_DESC(I, T, B, R) {T, B, R},
     TMND_S16_SHAPE_LIST(TMND_S16_DESC)
 #undef TMND_S16_DESC
 };
@@ -46,7 +46,7 @@ int per_sm(int shape) {
     if (dev < 0 || dev >= 64) dev = 0;
     if (!g_per_sm[dev][shape]) {
         switch (shape) {
-#define TMND_S16_OCC(I, T, B, P, R) \
+#define TMND_S16_OCC(I, T, B, R) \
     case I: g_per_sm[dev][I] = s16_per_sm_##I(); break;
             TMND_S16_SHAPE_LIST(TMND_S16_OCC)
 #undef TMND_S16_OCC
@@ -123,7 +123,7 @@ void launch_hop_even_s16(const Geom &g, const SiteTermF &st, const int2 *links, 
     bt.order = shape / NCOMPILED;
     const int nb = hop_blocks_s16(g, shape);
     switch (shape % NCOMPILED) {
-#define TMND_S16_EVEN(I, T, B, P, R) \
+#define TMND_S16_EVEN(I, T, B, R) \
     case I: s16_even_##I(g, st, links, in, out, dag, done, s, bt, nb); break;
         TMND_S16_SHAPE_LIST(TMND_S16_EVEN)
 #undef TMND_S16_EVEN
@@ -139,7 +139,7 @@ void launch_hop_odd_s16(const Geom &g, const SiteTermF &st, const int2 *links, S
     bt.order = shape / NCOMPILED;
     const int nb = hop_blocks_s16(g, shape);
     switch (shape % NCOMPILED) {
-#define TMND_S16_ODD(I, T, B, P, R) \
+#define TMND_S16_ODD(I, T, B, R) \
     case I: s16_odd_##I(g, st, links, psi, te, out, dag, epi, ea, s, bt, nb); break;
         TMND_S16_SHAPE_LIST(TMND_S16_ODD)
 #undef TMND_S16_ODD
@@ -316,7 +316,7 @@ extern "C" tmnd_status tmnd_s16_shape_info(int shape, int *threads, int *blocks_
     const ShapeDesc &d = kShapes[shape % NCOMPILED];
     if (threads) *threads = d.threads;
     if (blocks_per_sm) *blocks_per_sm = d.minb;
-    if (prefetch) *prefetch = d.pf;
+    if (prefetch) *prefetch = 1;  // every shape loads the next direction ahead
     if (order) *order = shape / NCOMPILED;
     return TMND_OK;
 }

@@ -11,7 +11,7 @@
 //   (1 + gamma_mu) psi = (chi,  B^+ chi),  chi = psi_up + B psi_lo
 // and only the two-spin chi is multiplied by the link (spin projection).
 //
-// Work split.  1152 FP64 multiply-adds per site took 768 clocks of an SM's FP64 pipe; as 3456 integer ones
+// Work split.  1152 FP64 multiply-adds per site take 576 clocks of an SM's FP64 pipe; as 3456 integer ones
 // they take 115, near the 100 that a site's ~2100 bytes take at the HBM rate.  A block of four warps works
 // on 16 sites: warp mu does the two hops of direction mu for both flavours (lanes 0..15 and 16..31), the
 // parts meet in shared memory, and warp s finishes spin s.  Against one thread per site and flavour for

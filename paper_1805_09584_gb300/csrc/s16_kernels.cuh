@@ -18,7 +18,7 @@
 // A block works on tiles of consecutive sites, a thread per site, flavour and one of RP right-hand sides:
 // lane bit 4 is the flavour, for RP = 2 bit 3 the right-hand side, the low bits the site.  The tile's eight
 // links per site are decoded once, row 2 included, into shared memory as FP32 and serve both flavours and
-// every right-hand side; the neighbours' words come straight from global memory (PF: those of the next
+// every right-hand side; the neighbours' words come straight from global memory (those of the next
 // direction are loaded before the current one is processed).  Arithmetic in s16_hop.cuh.
 // RP = 2 halves the shared-memory traffic for the links (a warp's 16-byte reads fall on 8 sites, one line,
 // instead of 16; with RP = 1 that traffic keeps the L1 data pipe 68 % busy): 7 % faster at 16^3x32 with 8 right-hand
@@ -42,10 +42,10 @@
 namespace {
 
 // Launch shapes the kernels are compiled in: threads per block, resident blocks per SM the register budget is
-// cut for, next-direction prefetch, right-hand sides per pass (0: the form of s16_site.cuh, a site per thread).  The
+// cut for, right-hand sides per pass (0: the form of s16_site.cuh, a site per thread).  The
 // autotuner times each on the GPU per (lattice, right-hand sides per launch) and keeps the fastest; shape 0 is the
 // default.
-#define TMND_S16_SHAPE_LIST(X) X(0, 128, 4, true, 1) X(1, 128, 5, true, 2) X(2, 64, 8, true, 2) X(3, 128, 3, true, 0)
+#define TMND_S16_SHAPE_LIST(X) X(0, 128, 4, 1) X(1, 128, 5, 2) X(2, 64, 8, 2) X(3, 128, 3, 0)
 
 template <int NT, int RP>
 struct Tile {
@@ -93,26 +93,23 @@ __device__ __forceinline__ void load_tile(const LatGeom &g, int apbc, const int2
     }
 }
 
-template <int D, bool G5IN, bool PF, int NT, int RP>
+template <int D, bool G5IN, int NT, int RP>
 __device__ __forceinline__ void hop_seq(const Tile<NT, RP> &t, int i, const S16In &in, int f, const Raw &cur, f2 up[3][2],
                                         f2 lo[3][2]) {
     Raw nxt;
-    if constexpr (PF && D < 7) load_raw(in, f, t.nb[D + 1][i], nxt);
+    if constexpr (D < 7) load_raw(in, f, t.nb[D + 1][i], nxt);
     f2 u[9];
     t.links.get(D, i, u);
     hop_dir<D / 2, (D & 1) ? -1 : 1, G5IN, D == 0>(cur, u, up, lo);
-    if constexpr (D < 7) {
-        if constexpr (!PF) load_raw(in, f, t.nb[D + 1][i], nxt);
-        hop_seq<D + 1, G5IN, PF, NT, RP>(t, i, in, f, nxt, up, lo);
-    }
+    if constexpr (D < 7) hop_seq<D + 1, G5IN, NT, RP>(t, i, in, f, nxt, up, lo);
 }
 // H psi at tile site i, flavour f: v[spin*3 + colour]
-template <bool G5IN, bool PF, int NT, int RP>
+template <bool G5IN, int NT, int RP>
 __device__ __forceinline__ void hop_all(const Tile<NT, RP> &t, int i, const S16In &in, int f, f2 v[12]) {
     f2 up[3][2], lo[3][2];
     Raw r;
     load_raw(in, f, t.nb[0][i], r);
-    hop_seq<0, G5IN, PF, NT, RP>(t, i, in, f, r, up, lo);
+    hop_seq<0, G5IN, NT, RP>(t, i, in, f, r, up, lo);
 #pragma unroll
     for (int c = 0; c < 3; c++) {
         v[c] = make_float2(up[c][0].x, up[c][1].x);
@@ -182,7 +179,7 @@ struct Place {
     }
 };
 
-template <bool DAG, bool PF, int NT, int MB, int RP>
+template <bool DAG, int NT, int MB, int RP>
 __global__ void __launch_bounds__(NT, MB) k_hop_even_s16(LatGeom g, int apbc, SiteTermF st, const int2 *__restrict__ links,
                                                          S16In in, S16Out out, const int *done, int ntile,
                                                          S16Batch bt) {
@@ -205,7 +202,7 @@ __global__ void __launch_bounds__(NT, MB) k_hop_even_s16(LatGeom g, int apbc, Si
         bool on = h < g.Vh;
         const int k = pl.rhs(k0, bt, on);
         f2 p[12], o[12];
-        hop_all<DAG, PF, NT, RP>(t, pl.i, s16_at(in, k * bt.stride), f, p);
+        hop_all<DAG, NT, RP>(t, pl.i, s16_at(in, k * bt.stride), f, p);
 #pragma unroll
         for (int q = 0; q < 12; q++) {
             const float b = q < 6 ? b0 : -b0;
@@ -220,7 +217,7 @@ __global__ void __launch_bounds__(NT, MB) k_hop_even_s16(LatGeom g, int apbc, Si
 // shared slot per (right-hand side, sum, pair of sites).  Of two sums the second flavour's lanes do the second, so
 // that both take one FP64 instruction of each kind.  Against FP32 sums over 4 or 8 sites (four launches of an
 // iteration, 8 right-hand sides): 32^3x64 4.33 -> 4.23 ms, 24^3x48 1.32 -> 1.30 ms, 16^3x32 298 -> 307 us.
-template <bool DAG, int EPI, bool PF, int NT, int MB, int RP>
+template <bool DAG, int EPI, int NT, int MB, int RP>
 __global__ void __launch_bounds__(NT, MB) k_hop_odd_s16(LatGeom g, int apbc, SiteTermF st, const int2 *__restrict__ links,
                                                         S16In psi_all, S16In te_all, S16Out out_all, S16EpiArgs ea,
                                                         int ntile, S16Batch bt) {
@@ -258,7 +255,7 @@ __global__ void __launch_bounds__(NT, MB) k_hop_odd_s16(LatGeom g, int apbc, Sit
         const S16In te = s16_at(te_all, k * bt.stride), psi = s16_at(psi_all, k * bt.stride);
         const int hc = min(h, Vh - 1);
         f2 v[12];
-        hop_all<false, PF, NT, RP>(t, pl.i, te, f, v);
+        hop_all<false, NT, RP>(t, pl.i, te, f, v);
         Raw own, oth;
         load_raw(psi, f, hc, own);
         load_raw(psi, 1 - f, hc, oth);
@@ -319,23 +316,23 @@ __global__ void __launch_bounds__(NT, MB) k_hop_odd_s16(LatGeom g, int apbc, Sit
     }
 }
 
-template <bool PF, int NT, int MB, int RP>
+template <int NT, int MB, int RP>
 int per_sm_of(int dev) {
     int a = 0, b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_hop_odd_s16<true, EPI_MMS_R, PF, NT, MB, RP>, NT, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_hop_even_s16<true, PF, NT, MB, RP>, NT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_hop_odd_s16<true, EPI_MMS_R, NT, MB, RP>, NT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_hop_even_s16<true, NT, MB, RP>, NT, 0);
     a = a < b ? a : b;
     (void)dev;
     return a > 0 ? a : 1;
 }
 
-template <bool PF, int NT, int MB, int RP>
+template <int NT, int MB, int RP>
 void launch_odd_shape(const Geom &g, const SiteTermF &st, const int2 *links, S16In psi, S16In te, S16Out out,
                       bool dag, HopEpi epi, const S16EpiArgs &ea, cudaStream_t s, const S16Batch &bt, int nb) {
     constexpr int SITES = Tile<NT, RP>::SITES;
     const int ntile = (g.Vh + SITES - 1) / SITES;
 #define TMND_ODD16(D, E) \
-    launch_dependent_if(ntile <= nb, k_hop_odd_s16<D, E, PF, NT, MB, RP>, dim3(nb), NT, s, lat_geom(g), g.apbc, st, links, psi, te, out, ea, ntile, bt)
+    launch_dependent_if(ntile <= nb, k_hop_odd_s16<D, E, NT, MB, RP>, dim3(nb), NT, s, lat_geom(g), g.apbc, st, links, psi, te, out, ea, ntile, bt)
     if (!dag) {
         switch (epi) {
             case EPI_STORE: TMND_ODD16(false, EPI_STORE); break;
@@ -358,19 +355,19 @@ void launch_odd_shape(const Geom &g, const SiteTermF &st, const int2 *links, S16
 
 // Launches overlap with the kernel before them only on lattices with at most a tile per block: where the blocks
 // fill the chip for several tiles, the waiting blocks of the next launch cost 2 % (8 right-hand sides, 24^3x48).
-// the extern entry points of one compiled shape (I, threads T, blocks per SM B, prefetch P)
-#define TMND_S16_DEFINE_SHAPE(I, T, B, P, R)                                                                     \
-    int s16_per_sm_##I() { return per_sm_of<P, T, B, R>(0); }                                                   \
+// the extern entry points of one compiled shape (I, threads T, blocks per SM B, right-hand sides per pass R)
+#define TMND_S16_DEFINE_SHAPE(I, T, B, R)                                                                        \
+    int s16_per_sm_##I() { return per_sm_of<T, B, R>(0); }                                                   \
     void s16_even_##I(const Geom &g, const SiteTermF &st, const int2 *links, S16In in, S16Out out, bool dag,    \
                       const int *done, cudaStream_t s, const S16Batch &bt, int nb) {                             \
         const LatGeom lg = lat_geom(g);                                                                          \
         const int sites = T / (2 * R), ntile = (g.Vh + sites - 1) / sites;                                       \
         if (dag)                                                                                                 \
-            launch_dependent_if(ntile <= nb, k_hop_even_s16<true, P, T, B, R>, dim3(nb), T, s, lg, g.apbc, st, links, in, out, done, ntile, bt);  \
+            launch_dependent_if(ntile <= nb, k_hop_even_s16<true, T, B, R>, dim3(nb), T, s, lg, g.apbc, st, links, in, out, done, ntile, bt);  \
         else                                                                                                     \
-            launch_dependent_if(ntile <= nb, k_hop_even_s16<false, P, T, B, R>, dim3(nb), T, s, lg, g.apbc, st, links, in, out, done, ntile, bt); \
+            launch_dependent_if(ntile <= nb, k_hop_even_s16<false, T, B, R>, dim3(nb), T, s, lg, g.apbc, st, links, in, out, done, ntile, bt); \
     }                                                                                                            \
     void s16_odd_##I(const Geom &g, const SiteTermF &st, const int2 *links, S16In psi, S16In te, S16Out out,     \
                      bool dag, HopEpi epi, const S16EpiArgs &ea, cudaStream_t s, const S16Batch &bt, int nb) {   \
-        launch_odd_shape<P, T, B, R>(g, st, links, psi, te, out, dag, epi, ea, s, bt, nb);                      \
+        launch_odd_shape<T, B, R>(g, st, links, psi, te, out, dag, epi, ea, s, bt, nb);                      \
     }

@@ -14,6 +14,7 @@
 // neighbours' latency together.
 #pragma once
 
+#include "launch.cuh"
 #include "s16_kernels.cuh"
 
 namespace {
@@ -135,25 +136,22 @@ __device__ __forceinline__ void load_dir(const S16In &in, const int2 *__restrict
     load_raw2(in, nb.n[D], r.f);
     load_link(links + ((size_t)par * 4 + D / 2) * 3 * Vh, (D & 1) ? nb.n[D] : h, r.l);
 }
-template <int P, int D, bool G5IN, bool PF>
+template <int P, int D, bool G5IN>
 __device__ __forceinline__ void site_seq(const S16In &in, const int2 *__restrict__ links, int Vh, int h, const Nbr<P> &nb,
                                          const SiteRaw &cur, f2 acc[4][3][2]) {
     SiteRaw nxt;
-    if constexpr (PF && D < 7) load_dir<P, D + 1>(in, links, Vh, h, nb, nxt);
+    if constexpr (D < 7) load_dir<P, D + 1>(in, links, Vh, h, nb, nxt);
     site_dir<D / 2, (D & 1) ? -1 : 1, G5IN, D == 0>(cur, D == 0 ? nb.sf : D == 1 ? nb.sb : 1.0f, acc);
-    if constexpr (D < 7) {
-        if constexpr (!PF) load_dir<P, D + 1>(in, links, Vh, h, nb, nxt);
-        site_seq<P, D + 1, G5IN, PF>(in, links, Vh, h, nb, nxt, acc);
-    }
+    if constexpr (D < 7) site_seq<P, D + 1, G5IN>(in, links, Vh, h, nb, nxt, acc);
 }
 // H psi at site h
-template <int P, bool G5IN, bool PF>
+template <int P, bool G5IN>
 __device__ __forceinline__ void site_hop(const LatGeom &g, int apbc, const S16In &in, const int2 *__restrict__ links, int h,
                                          f2 acc[4][3][2]) {
     const Nbr<P> nb(g, apbc, h);
     SiteRaw r;
     load_dir<P, 0>(in, links, g.Vh, h, nb, r);
-    site_seq<P, 0, G5IN, PF>(in, links, g.Vh, h, nb, r, acc);
+    site_seq<P, 0, G5IN>(in, links, g.Vh, h, nb, r, acc);
 }
 
 // quantise and store a site
@@ -194,7 +192,7 @@ __device__ __forceinline__ void site_walk(int Vh, const S16Batch &bt, F &&site) 
         }
 }
 
-template <bool DAG, bool PF, int NT, int MB>
+template <bool DAG, int NT, int MB>
 __global__ void __launch_bounds__(NT, MB) k_site_even_s16(LatGeom g, int apbc, SiteTermF st, const int2 *__restrict__ links,
                                                           S16In in, S16Out out, const int *done, S16Batch bt) {
     dependent_begin();
@@ -202,7 +200,7 @@ __global__ void __launch_bounds__(NT, MB) k_site_even_s16(LatGeom g, int apbc, S
     const float a = st.kappa2 * st.inv_det, e = a * st.kpp;
     site_walk<NT>(g.Vh, bt, [&](int h, int k) {
         f2 acc[4][3][2];
-        site_hop<0, DAG, PF>(g, apbc, s16_at(in, k * bt.stride), links, h, acc);
+        site_hop<0, DAG>(g, apbc, s16_at(in, k * bt.stride), links, h, acc);
         f2 o[4][3][2];
 #pragma unroll
         for (int s = 0; s < 4; s++) {
@@ -220,7 +218,7 @@ __global__ void __launch_bounds__(NT, MB) k_site_even_s16(LatGeom g, int apbc, S
 
 // Reduction partials: a flavour's squares in FP32, the site's sum added in FP64 to the thread's own slot of dynamic
 // shared memory, [right-hand side][sum][thread].
-template <bool DAG, int EPI, bool PF, int NT, int MB>
+template <bool DAG, int EPI, int NT, int MB>
 __global__ void __launch_bounds__(NT, MB) k_site_odd_s16(LatGeom g, int apbc, SiteTermF st, const int2 *__restrict__ links,
                                                          S16In psi_all, S16In te_all, S16Out out_all, S16EpiArgs ea,
                                                          S16Batch bt) {
@@ -236,7 +234,7 @@ __global__ void __launch_bounds__(NT, MB) k_site_odd_s16(LatGeom g, int apbc, Si
     const float kp = DAG ? -st.kp : st.kp;
     site_walk<NT>(Vh, bt, [&](int h, int k) {
         f2 acc[4][3][2];
-        site_hop<1, false, PF>(g, apbc, s16_at(te_all, k * bt.stride), links, h, acc);
+        site_hop<1, false>(g, apbc, s16_at(te_all, k * bt.stride), links, h, acc);
         const S16In psi = s16_at(psi_all, k * bt.stride), aux = s16_at(ea.aux, k * bt.stride);
         const float sigma = (float)(EPI == EPI_MMS_R && ea.per_rhs_sigma ? ea.sigma_k[k] : ea.sigma);
         const float alpha = EPI == EPI_MMS_R ? (float)ea.alpha[(size_t)k * ea.alpha_stride] : 0.0f;
@@ -312,22 +310,22 @@ __global__ void __launch_bounds__(NT, MB) k_site_odd_s16(LatGeom g, int apbc, Si
         }
 }
 
-template <bool PF, int NT, int MB>
+template <int NT, int MB>
 int site_per_sm() {
     int a = 0, b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_site_odd_s16<true, EPI_MMS_R, PF, NT, MB>, NT, sizeof(double) * 2 * NT);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_site_even_s16<true, PF, NT, MB>, NT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_site_odd_s16<true, EPI_MMS_R, NT, MB>, NT, sizeof(double) * 2 * NT);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_site_even_s16<true, NT, MB>, NT, 0);
     a = a < b ? a : b;
     return a > 0 ? a : 1;
 }
 
-template <bool PF, int NT, int MB>
+template <int NT, int MB>
 void launch_site_odd(const Geom &g, const SiteTermF &st, const int2 *links, S16In psi, S16In te, S16Out out, bool dag,
                      HopEpi epi, const S16EpiArgs &ea, cudaStream_t s, const S16Batch &bt, int nb) {
     const int ntile = (g.Vh + NT - 1) / NT;
     static_assert(sizeof(double) * 2 * TMND_MAX_BATCH * NT <= 46 * 1024, "partials fit the default shared memory");
 #define TMND_SITE16(D, E)                                                                                       \
-    launch_dependent_smem(ntile <= nb, k_site_odd_s16<D, E, PF, NT, MB>, dim3(nb), NT,                          \
+    launch_dependent_smem(ntile <= nb, k_site_odd_s16<D, E, NT, MB>, dim3(nb), NT,                          \
                           E == EPI_STORE_NORMS ? sizeof(double) * 2 * bt.nrhs * NT                              \
                                                : E == EPI_MMS_R ? sizeof(double) * bt.nrhs * NT : (size_t)0,   \
                           s, lat_geom(g), g.apbc, st, links, psi, te, out, ea, bt)
@@ -342,18 +340,18 @@ void launch_site_odd(const Geom &g, const SiteTermF &st, const int2 *links, S16I
 
 }  // namespace
 
-// the extern entry points of a shape of this form (I, threads T, blocks per SM B, prefetch P)
-#define TMND_S16_DEFINE_SITE_SHAPE(I, T, B, P)                                                                   \
-    int s16_per_sm_##I() { return site_per_sm<P, T, B>(); }                                                     \
+// the extern entry points of a shape of this form (I, threads T, blocks per SM B)
+#define TMND_S16_DEFINE_SITE_SHAPE(I, T, B)                                                                      \
+    int s16_per_sm_##I() { return site_per_sm<T, B>(); }                                                     \
     void s16_even_##I(const Geom &g, const SiteTermF &st, const int2 *links, S16In in, S16Out out, bool dag,    \
                       const int *done, cudaStream_t s, const S16Batch &bt, int nb) {                             \
         const int ntile = (g.Vh + T - 1) / T;                                                                    \
         if (dag)                                                                                                 \
-            launch_dependent_if(ntile <= nb, k_site_even_s16<true, P, T, B>, dim3(nb), T, s, lat_geom(g), g.apbc, st, links, in, out, done, bt);  \
+            launch_dependent_if(ntile <= nb, k_site_even_s16<true, T, B>, dim3(nb), T, s, lat_geom(g), g.apbc, st, links, in, out, done, bt);  \
         else                                                                                                     \
-            launch_dependent_if(ntile <= nb, k_site_even_s16<false, P, T, B>, dim3(nb), T, s, lat_geom(g), g.apbc, st, links, in, out, done, bt); \
+            launch_dependent_if(ntile <= nb, k_site_even_s16<false, T, B>, dim3(nb), T, s, lat_geom(g), g.apbc, st, links, in, out, done, bt); \
     }                                                                                                            \
     void s16_odd_##I(const Geom &g, const SiteTermF &st, const int2 *links, S16In psi, S16In te, S16Out out,     \
                      bool dag, HopEpi epi, const S16EpiArgs &ea, cudaStream_t s, const S16Batch &bt, int nb) {   \
-        launch_site_odd<P, T, B>(g, st, links, psi, te, out, dag, epi, ea, s, bt, nb);                          \
+        launch_site_odd<T, B>(g, st, links, psi, te, out, dag, epi, ea, s, bt, nb);                          \
     }
