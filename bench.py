@@ -103,13 +103,12 @@ S16_SPINOR_BYTES_PER_SITE = 2 * (200 + 300) + 100
 # 192 + 8 x 72 + 192, odd launch + psi 192, the sigma term's 192
 F32_Q2_BYTES_PER_SITE = 2 * ((192 + 576 + 192) + (192 + 192 + 576 + 192)) + 192
 S16_LINK_BYTES_PER_SITE = 4 * 192
-# DRAM bytes (read + write) of one 16-bit Qhat^2 + sigma, one ncu capture of its 4 launches:
+# DRAM bytes (read + write) of one 16-bit Qhat^2 + sigma at 24^3x48, one ncu capture of its 4 launches
+# (k_site_*_s16 at one right-hand side, k_hop_*_s16 in grid-stride order at 8):
 # {(lattice V/2, RHS per launch): bytes}
-# (of the kernel's earlier form, both flavours per thread; the 8-RHS entry in grid-stride order)
-S16_Q2_TRAFFIC = {(331776, 1): (97.503232e6 + 3.967232e6) + (132.547840e6 + 8.404480e6)
-                  + (97.519360e6 + 3.632896e6) + (169.893632e6 + 15.372288e6),
-                  (1048576, 8): (3218.8e6 + 820.7e6) + (4144.8e6 + 821.5e6)
-                  + (3223.5e6 + 816.4e6) + (4910.6e6 + 823.1e6)}
+S16_Q2_TRAFFIC = {(331776, 1): (97.10e6 + 4.29e6) + (131.46e6 + 6.01e6) + (97.00e6 + 2.65e6) + (165.11e6 + 11.51e6),
+                  (331776, 8): (507.95e6 + 243.43e6) + (688.15e6 + 245.86e6) + (509.26e6 + 238.50e6)
+                  + (1008.16e6 + 247.91e6)}
 
 
 def _dist():
@@ -295,7 +294,7 @@ def s16_roofline(tm, g, flush, stream, nrhs=1, reps=20):
                     + (", scaled by the number of sites" if vh != g.vh else ""))
             break
     del q, o
-    return {"bound": "hbm", "kernel": f"k_hop_even_s16/k_hop_odd_s16 (16-bit stencil, Qhat^2 + sigma: 4 launches, "
+    return {"bound": "hbm", "kernel": f"{'k_site' if nrhs == 1 else 'k_hop'}_even_s16/odd_s16 (16-bit stencil, Qhat^2 + sigma: 4 launches, "
                                       f"{nrhs} RHS per launch)",
             "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak, "traffic": tr,
             "traffic_note": note, "algorithmic_bytes": byts, "peak_source": src_peak,
@@ -424,8 +423,8 @@ def run_form(args):
                       "shape_mms": shm, "ms_mms": [round(float(v), 4) for v in tmm]}
         extra["autotune"] = {"shapes": [tm.tmnd_s16_shape_info(i) for i in range(tm.S16_SHAPES)],
                              "shape_fields": ["threads per block", "blocks per SM", "next-direction prefetch",
-                                              "loop order (0 chunk, sites outside; 1 chunk, RHS outside; "
-                                              "2 grid stride, sites outside; 3 grid stride over (32-site group, RHS) per warp)"],
+                                              "loop order (0 own tiles, tiles outside; 1 own tiles, RHS outside; "
+                                              "2 grid stride, tiles outside; 3 grid stride over (tile, RHS) items)"],
                              "per_nrhs": per, "s": time.perf_counter() - t0}
     if args.form == "hybrid":
         t0 = time.perf_counter()

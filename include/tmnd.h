@@ -138,12 +138,12 @@ tmnd_status tmnd_spinor_unpack(const tmnd_gauge *g, void *dev_canonical, const v
  * intermediates rounded to 16 bits per site); then 1 <= nrhs <= 16 and every
  * stencil launch covers all nrhs right-hand sides (the links are read once per
  * launch and shared through the cache).  With TMND_OP_F32 in `op`, in and out
- * are TMND_F32 spinors and the operator is the FP32 one (one right-hand side
- * per launch sequence).  `out` and `in` must not overlap.  Uses
- * the handle's workspace (one even-site and one odd-site spinor per right-hand
- * side for TMND_OP_S16; one of each for TMND_OP_F32, and for FP64 spinors on
- * lattices that fill the chip: smaller ones get up to ~25000 sites' worth of
- * each and run several right-hand sides per launch), growing it on first use.
+ * are TMND_F32 spinors and the operator is the FP32 one.  `out` and `in` must
+ * not overlap.  Uses the handle's workspace (one even-site and one odd-site
+ * spinor per right-hand side for TMND_OP_S16; for FP32 and FP64 spinors one of
+ * each on lattices that fill the chip, up to ~25000 sites' worth of each on
+ * smaller ones, which run several right-hand sides per launch), growing it on
+ * first use.
  * (Sec. 2 even-odd Schur complement; Eq. "g5tau1-hermiticity".) */
 tmnd_status tm_nd_apply(tmnd_gauge *g, void *out, const void *in, int op, double sigma,
                         int nrhs, void *stream);
@@ -185,7 +185,7 @@ tmnd_status tm_nd_apply_noalloc(const tmnd_gauge *g, void *out, const void *in, 
 
 /* Launch-shape autotuner of the sloppy (16-bit) stencil.  Its kernels run in
  * TMND_S16_SHAPES launch variants: 4 compiled shapes (threads per block x resident blocks
- * per SM the register budget is cut for x next-direction prefetch; shape 0 takes one right-hand
+ * per SM the register budget is cut for; shape 0 takes one right-hand
  * side per pass over a block's tile of sites, 1 and 2 take two; shape 3 has a thread per site and no
  * tiles, for one right-hand side; its orders 1 and 3 are 0 and 2) x 4 loop orders (0: every
  * block walks its own tiles, all right-hand sides of a tile in turn; 1: its tiles
@@ -211,7 +211,7 @@ tmnd_status tmnd_autotune_mms(tmnd_gauge *g, int nrhs, int *shape_out, double *m
 /* Use shape `shape` for every later 16-bit stencil launch of this process (-1: back to the
  * tuned choice).  For tests and measurements; results do not depend on the shape. */
 tmnd_status tmnd_s16_force_shape(int shape);
-/* Threads per block, resident blocks per SM, prefetch flag (0/1) and loop order (0..3 as
+/* Threads per block, resident blocks per SM, prefetch flag (1 in every variant) and loop order (0..3 as
  * above) of a variant (NULL outputs skipped). */
 tmnd_status tmnd_s16_shape_info(int shape, int *threads, int *blocks_per_sm, int *prefetch, int *order);
 
