@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_prolong(TrGeom g, const float2 *
     const int nr = min(NC / 2, nrhs - rhs0);
     const int len = g.nsb * 6;
     const size_t Vh = g.Vh;
-    for (int i = threadIdx.x; i < g.nv * NC; i += TR_THREADS) {
+    for (int i = threadIdx.x; i < g.nv * NC; i += blockDim.x) {
         const int k = i / NC, col = i - k * NC;
         sc[k][col] = col < 2 * nr ? in[(((size_t)(rhs0 + (col >> 1)) * g.nblock + b) * 2 + (col & 1)) * 2 * g.nv +
                                        chi * g.nv + k]
@@ -203,21 +203,24 @@ __global__ void __launch_bounds__(TR_THREADS) k_prolong(TrGeom g, const float2 *
     __syncthreads();
     const float2 *Pb = P + (size_t)blockIdx.x * ((size_t)g.nv * len);
     const int4 o = corner(g, b);
-    for (int p = threadIdx.x; p < len / 2; p += TR_THREADS) {
+    for (int p = threadIdx.x; p < len / 2; p += blockDim.x) {
         int i0, i1, s, c, par, h;
         pair_of<ZPAIR>(p, i0, i1, s, c);
         float2 acc[2][NC];
 #pragma unroll
         for (int j = 0; j < NC; j++) acc[0][j] = acc[1][j] = make_float2(0.f, 0.f);
-        if (p + TR_THREADS < len / 2) {  // the next pair's elements on their way
+        if (p + blockDim.x < len / 2) {  // the next pair's elements on their way
             int n0, n1, ns, nc;
-            pair_of<ZPAIR>(p + TR_THREADS, n0, n1, ns, nc);
+            pair_of<ZPAIR>(p + blockDim.x, n0, n1, ns, nc);
             for (int k = 0; k < g.nv; k++) {
                 prefetch_l1(&Pb[(size_t)k * len + n0]);
                 if (ZPAIR) prefetch_l1(&Pb[(size_t)k * len + n1]);
             }
         }
-#pragma unroll 4
+        // few columns leave the loads' latency bare: 8 vectors' elements in flight, 4 where the sums need the registers
+        // (24 vectors, 16^3x32: 1 right-hand side 128 -> 108 us, 2 126 -> 108 us; 2^4 aggregates, 8 vectors, 16x8^3, 2
+        // right-hand sides 23.4 -> 17.4 us, with both changes)
+#pragma unroll(NC <= 4 ? 8 : 4)
         for (int k = 0; k < g.nv; k++) {
             const float2 a0 = __ldg(&Pb[(size_t)k * len + i0]), a1 = __ldg(&Pb[(size_t)k * len + i1]);
 #pragma unroll
@@ -292,8 +295,11 @@ template <int NC>
 cudaError_t start_prolong(const TrGeom &g, const float2 *P, const float2 *in, float2 *v, int nrhs, bool zpair,
                           cudaStream_t s) {
     const dim3 grid(2 * g.nblock, (nrhs + NC / 2 - 1) / (NC / 2));
-    if (zpair) k_prolong<NC, true><<<grid, TR_THREADS, 0, s>>>(g, P, in, v, nrhs);
-    else k_prolong<NC, false><<<grid, TR_THREADS, 0, s>>>(g, P, in, v, nrhs);
+    // no more threads than pairs: 2^4 aggregates have 48 (16^3x32, 8 vectors, 8 right-hand sides: blocks of 256
+    // 228 us, of 64 185 us)
+    const int pairs = g.nsb * 3, threads = pairs < TR_THREADS ? (pairs + 31) & ~31 : TR_THREADS;
+    if (zpair) k_prolong<NC, true><<<grid, threads, 0, s>>>(g, P, in, v, nrhs);
+    else k_prolong<NC, false><<<grid, threads, 0, s>>>(g, P, in, v, nrhs);
     return cudaGetLastError();
 }
 
